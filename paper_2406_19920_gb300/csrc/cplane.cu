@@ -44,7 +44,7 @@ template <typename T, int NX, int NZ, int C> struct ClusterCfg {
   static constexpr size_t xbytes = (size_t)CP * pair_bytes > (size_t)CW * col_bytes ? (size_t)CP * pair_bytes
                                                                                     : (size_t)CW * col_bytes;
   static constexpr size_t bytes = fixed + xbytes;
-  static constexpr int J3 = N2X / 2 + 1;
+  static constexpr int J3 = N2X / 2;
   static constexpr int JMAX0 = CP * N1X > CP * J3 ? CP * N1X : CP * J3;
   static constexpr int JMAX = JMAX0 > CW * N1Z ? JMAX0 : CW * N1Z;
   static constexpr int THREADS = JMAX >= 1024 ? 1024 : (JMAX + 31) / 32 * 32;
@@ -53,7 +53,7 @@ template <typename T, int NX, int NZ, int C> struct ClusterCfg {
 template <typename T, int NX, int NZ, int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(ClusterCfg<T, NX, NZ, C>::THREADS)
 k_cplane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__ twx,
-             const cplx<T> *__restrict__ twz, T in_scale, double *zrhs) {
+             const cplx<T> *__restrict__ twz, double *zrhs) {
   using Cfg = ClusterCfg<T, NX, NZ, C>;
   constexpr int P = Cfg::P, R = Cfg::R, PC = Cfg::PC, N1X = Cfg::N1X, XPITCH = Cfg::XPITCH;
   constexpr int N1Z = Cfg::N1Z, N2Z = Cfg::N2Z, CP = Cfg::CP, CW = Cfg::CW, J3 = Cfg::J3, NT = Cfg::THREADS;
@@ -79,7 +79,7 @@ k_cplane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict_
     const int np = min(CP, R / 2 - p0);
     for (int job = tid; job < np * N1X; job += NT) {
       const int p = job / N1X, n1 = job - p * N1X;
-      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, in_scale, n1, tw2x, X + (p * N1X + n1) * XPITCH);
+      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, n1, tw2x, X + (p * N1X + n1) * XPITCH);
     }
     __syncthreads();
     for (int job = tid; job < np * J3; job += NT) {
@@ -112,7 +112,7 @@ k_cplane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict_
       const int k2 = job / CW, c = job - k2 * CW;
       if (c < nc) {
         const cplx<T> u0 = col_step3<T, NZ, false, CW>(X, c, k2, dst + c0 + c, P);
-        if (zrhs && c0 + c == 0 && k2 == 0) zrhs[j] = (double)u0.x;
+        if (zrhs && c0 + c == 0 && k2 == 0) zrhs[j] = 0.5 * (double)u0.x;
       }
     }
     __syncthreads();
@@ -151,7 +151,7 @@ k_cplane_inv(Ptr3<cplx<T> *> S_, Ptr3<T *> out_, Ptr3<const T *> add_, const cpl
   cluster.sync();
   // z: own columns from HBM, results into the owner CTAs' rows
   const cplx<T> *srcS = S + (size_t)j * NZ * P;
-  const cplx<T> z0 = zsol ? mk<T>((T)zsol[j], (T)0) : mk<T>((T)0, (T)0);
+  const cplx<T> z0 = zsol ? mk<T>((T)(2.0 * zsol[j]), (T)0) : mk<T>((T)0, (T)0);
   const int cbeg = r * PC, cend = min(P, cbeg + PC);
   for (int c0 = cbeg; c0 < cend; c0 += CW) {
     const int nc = min(CW, cend - c0);
@@ -211,14 +211,14 @@ template <typename T> bool cplane_supported(int nx, int nz, int C) {
 
 template <typename T>
 cudaError_t launch_cplane_forward(const TransformGeom &g, int C, Ptr3<const T *> in, Ptr3<cplx<T> *> S,
-                                  const cplx<T> *twx, const cplx<T> *twz, T in_scale, cudaStream_t st) {
+                                  const cplx<T> *twx, const cplx<T> *twz, cudaStream_t st) {
 #define X(a, b, c)                                                                              \
   if (g.nx == a && g.nz == b && C == c) {                                                       \
     if constexpr (ClusterCfg<T, a, b, c>::ok) {                                                 \
       using Cfg = ClusterCfg<T, a, b, c>;                                                       \
       { cudaError_t e = ensure_max_smem<k_cplane_fwd<T, a, b, c>>(); if (e) return e; }          \
       IBM_KTRY(launch_pdl(k_cplane_fwd<T, a, b, c>, dim3(g.ny * c, g.nb), Cfg::THREADS, Cfg::bytes, st, in, S, \
-                          twx, twz, in_scale, g.zrhs));                                         \
+                          twx, twz, g.zrhs));                                                   \
       return cudaSuccess;                                                                       \
     }                                                                                           \
   }
@@ -237,7 +237,7 @@ cudaError_t launch_cplane_inverse(const TransformGeom &g, int C, Ptr3<cplx<T> *>
       using Cfg = ClusterCfg<T, a, b, c>;                                                       \
       { cudaError_t e = ensure_max_smem<k_cplane_inv<T, a, b, c>>(); if (e) return e; }          \
       IBM_KTRY(launch_pdl(k_cplane_inv<T, a, b, c>, dim3(g.ny * c, g.nb), Cfg::THREADS, Cfg::bytes, st, S, out, \
-                          addend, twx, twz, scale, g.zsol));                                    \
+                          addend, twx, twz, (T)0.5 * scale, g.zsol));                                    \
       return cudaSuccess;                                                                       \
     }                                                                                           \
   }
@@ -249,9 +249,9 @@ cudaError_t launch_cplane_inverse(const TransformGeom &g, int C, Ptr3<cplx<T> *>
 template bool cplane_supported<float>(int, int, int);
 template bool cplane_supported<double>(int, int, int);
 template cudaError_t launch_cplane_forward<float>(const TransformGeom &, int, Ptr3<const float *>, Ptr3<float2 *>,
-                                                  const float2 *, const float2 *, float, cudaStream_t);
+                                                  const float2 *, const float2 *, cudaStream_t);
 template cudaError_t launch_cplane_forward<double>(const TransformGeom &, int, Ptr3<const double *>,
-                                                   Ptr3<double2 *>, const double2 *, const double2 *, double,
+                                                   Ptr3<double2 *>, const double2 *, const double2 *,
                                                    cudaStream_t);
 template cudaError_t launch_cplane_inverse<float>(const TransformGeom &, int, Ptr3<float2 *>, Ptr3<float *>,
                                                   Ptr3<const float *>, const float2 *, const float2 *, float,

@@ -230,10 +230,10 @@ __device__ __forceinline__ void dft_epilogue(DftHdr *hdr, uint32_t tmem, uint32_
   }
 }
 
-// Forward: in (ny planes of nz x nx reals, times in_scale) -> S [ny][nz][P].
+// Forward: in (ny planes of nz x nx reals) -> S [ny][nz][P].
 __global__ void __launch_bounds__(kDftThreads, 1)
 k_dft_fwd(DftShape d, int ny, Ptr3<const float *> in_, Ptr3<float2 *> S_, const float *__restrict__ tab,
-          float in_scale, double *zrhs, int *err) {
+          double *zrhs, int *err) {
   extern __shared__ __align__(128) unsigned char smem[];
   DftHdr *hdr = reinterpret_cast<DftHdr *>(smem);
   unsigned char *R1 = smem + kHdr, *R2 = R1 + d.r1f, *R3 = R2 + d.r2f;
@@ -273,10 +273,10 @@ k_dft_fwd(DftShape d, int ny, Ptr3<const float *> in_, Ptr3<float2 *> S_, const 
           const int r = e / q4n, q4 = e - r * q4n;
           const uint32_t o = (uint32_t)(r >> 3) * sbo_x + (uint32_t)q4 * kLboPad + (uint32_t)(r & 7) * 16u;
           float4 h, l;
-          tf32_split(xv[it].x * in_scale, h.x, l.x);
-          tf32_split(xv[it].y * in_scale, h.y, l.y);
-          tf32_split(xv[it].z * in_scale, h.z, l.z);
-          tf32_split(xv[it].w * in_scale, h.w, l.w);
+          tf32_split(xv[it].x, h.x, l.x);
+          tf32_split(xv[it].y, h.y, l.y);
+          tf32_split(xv[it].z, h.z, l.z);
+          tf32_split(xv[it].w, h.w, l.w);
           *reinterpret_cast<float4 *>(Ah + o) = h;
           *reinterpret_cast<float4 *>(Al + o) = l;
         }
@@ -589,14 +589,13 @@ static int dft_grid_cap() {
   return cap;
 }
 
-cudaError_t launch_dft_forward(const TransformGeom &g, Ptr3<const float *> in, Ptr3<float2 *> S, float in_scale,
-                               cudaStream_t st) {
+cudaError_t launch_dft_forward(const TransformGeom &g, Ptr3<const float *> in, Ptr3<float2 *> S, cudaStream_t st) {
   if (!g.dft_fwd || !dft_tc_supported(g.nx, g.nz)) return cudaErrorNotSupported;
   const DftShape d = dft_shape(g.nx, g.ny, g.nz);
   IBM_KTRY(ensure_max_smem<k_dft_fwd>());
   const dim3 grid((unsigned)std::min(d.ngroups, dft_grid_cap()), (unsigned)g.nb);
   return launch_pdl(k_dft_fwd, grid, dim3(kDftThreads), kHdr + d.r1f + d.r2f + d.r3f, st, d, g.ny, in, S,
-                    (const float *)g.dft_fwd, in_scale, g.zrhs, g.err);
+                    (const float *)g.dft_fwd, g.zrhs, g.err);
 }
 
 cudaError_t launch_dft_inverse(const TransformGeom &g, Ptr3<float2 *> S, Ptr3<float *> out,

@@ -191,51 +191,84 @@ __device__ __forceinline__ void load_step_twiddles(cplx<T> *tw2, const cplx<T> *
 // ---------------------------------------------------------------------------
 
 // Rows forward, step 1, lane n1 of one real row pair (a = rows[0, N),
-// b = rows[N, 2N)): z = s (a + i b); x = the lane's exchange row (N2 entries).
+// b = rows[N, 2N)): z = a + i b; x = the lane's exchange row (N2 entries).
 template <typename T, int N>
-__device__ __forceinline__ void rfwd_step1(const T *rows, T s, int n1, const cplx<T> *tw2, cplx<T> *x) {
+__device__ __forceinline__ void rfwd_step1(const T *rows, int n1, const cplx<T> *tw2, cplx<T> *x) {
   constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
   cplx<T> v[N2];
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) v[n2] = mk<T>(rows[n1 + N1 * n2] * s, rows[N + n1 + N1 * n2] * s);
+  for (int n2 = 0; n2 < N2; ++n2) v[n2] = mk<T>(rows[n1 + N1 * n2], rows[N + n1 + N1 * n2]);
   reg_dft<false, N2>(v);
   x[0] = v[0];
 #pragma unroll
   for (int k2 = 1; k2 < N2; ++k2) x[k2] = cmul(v[k2], tw2[k2 * N1 + n1]);
 }
 
-// Rows forward, step 3, job q in [0, N2/2] of one pair (xp: the pair's
-// exchange rows, pitch PITCH): the columns q and N2 - q give Z_k and Z_{N-k}
-// together; writes A_k to dA[k] and B_k to dB[k] for its k <= N/2.
+// The two half spectra of a row pair from Z_k and Z_{N-k}, twice over:
+// 2 A_k = Z_k + conj Z_{N-k} to *a, 2 B_k = -i (Z_k - conj Z_{N-k}) to *b.
+// The factor 2 is a power of two (no rounding) that the inverse's scale takes
+// out again: 4 multiplications a bin less, which FP64 pays in full.
+template <typename C> __device__ __forceinline__ void split_put(C zk, C zn, C *a, C *b) {
+  using T = decltype(zk.x);
+  *a = mk<T>(zk.x + zn.x, zk.y - zn.y);
+  *b = mk<T>(zk.y + zn.y, zn.x - zk.x);
+}
+
+// Rows forward, step 3, of one pair (xp: the pair's exchange rows, pitch
+// PITCH): the columns q and N2 - q give Z_k and Z_{N-k} together, and the two
+// columns that are their own mirror image, 0 and N2/2, go together, so that
+// the N2/2 jobs of a pair (qa = q, qb) do the same work and a warp never runs
+// one job's branch with the other jobs' lanes idle.  Writes 2 A_k to dA[k]
+// and 2 B_k to dB[k].
 template <typename T, int N, int PITCH>
 __device__ __forceinline__ void rfwd_step3(const cplx<T> *xp, int q, cplx<T> *dA, cplx<T> *dB) {
   constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
-  const T h = (T)0.5;
-  auto put = [&](int k, cplx<T> zk, cplx<T> zn) {
-    dA[k] = mk<T>(h * (zk.x + zn.x), h * (zk.y - zn.y));
-    dB[k] = mk<T>(h * (zk.y + zn.y), -h * (zk.x - zn.x));
-  };
-  cplx<T> u[N1];
+  const bool own = q == 0;
+  const int qb = own ? N2 / 2 : N2 - q;
+  cplx<T> u[N1], w[N1];
 #pragma unroll
   for (int n1 = 0; n1 < N1; ++n1) u[n1] = xp[n1 * PITCH + q];
   reg_dft<false, N1>(u);
-  if (q == 0) {  // k = N2 k1, partner N2 (N1 - k1)
 #pragma unroll
-    for (int k1 = 0; k1 <= N1 / 2; ++k1) put(N2 * k1, u[k1], u[(N1 - k1) % N1]);
-  } else if (q == N2 / 2) {  // k = N2/2 + N2 k1, partner N2/2 + N2 (N1 - 1 - k1)
+  for (int n1 = 0; n1 < N1; ++n1) w[n1] = xp[n1 * PITCH + qb];
+  reg_dft<false, N1>(w);
 #pragma unroll
-    for (int k1 = 0; k1 < N1 / 2; ++k1) put(q + N2 * k1, u[k1], u[N1 - 1 - k1]);
-  } else {
-    cplx<T> w[N1];
-#pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) w[n1] = xp[n1 * PITCH + (N2 - q)];
-    reg_dft<false, N1>(w);
-#pragma unroll
-    for (int k1 = 0; k1 < N1 / 2; ++k1) {
-      put(q + N2 * k1, u[k1], w[N1 - 1 - k1]);
-      put(N2 - q + N2 * k1, w[k1], u[N1 - 1 - k1]);
-    }
+  for (int k1 = 0; k1 < N1 / 2; ++k1) {
+    const cplx<T> zu = own ? u[(N1 - k1) % N1] : w[N1 - 1 - k1];
+    const cplx<T> zw = own ? w[N1 - 1 - k1] : u[N1 - 1 - k1];
+    split_put(u[k1], zu, dA + q + N2 * k1, dB + q + N2 * k1);
+    split_put(w[k1], zw, dA + qb + N2 * k1, dB + qb + N2 * k1);
   }
+  if (own) split_put(u[N1 / 2], u[N1 / 2], dA + N / 2, dB + N / 2);
+}
+
+// The same with one column per thread: the threads t = 2 i, 2 i + 1 of a pair
+// (neighbouring lanes) take the two columns of job i and swap the halves that
+// the other one needs.  Every lane of the warp calls it (live: the lane has a
+// job).
+template <typename T, int N, int PITCH>
+__device__ __forceinline__ void rfwd_step3_lane(const cplx<T> *xp, int t, bool live, cplx<T> *dA, cplx<T> *dB) {
+  constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
+  const int i = t >> 1;
+  const bool odd = t & 1, own = i == 0;
+  const int col = !odd ? i : own ? N2 / 2 : N2 - i;
+  cplx<T> u[N1];
+#pragma unroll
+  for (int n1 = 0; n1 < N1; ++n1) u[n1] = xp[n1 * PITCH + col];
+  reg_dft<false, N1>(u);
+  cplx<T> zn[N1 / 2];
+#pragma unroll
+  for (int k1 = 0; k1 < N1 / 2; ++k1) {
+    const cplx<T> mine = odd ? u[N1 - 1 - k1] : u[(N1 - k1) % N1];
+    cplx<T> theirs;
+    theirs.x = __shfl_xor_sync(0xffffffffu, u[N1 - 1 - k1].x, 1);
+    theirs.y = __shfl_xor_sync(0xffffffffu, u[N1 - 1 - k1].y, 1);
+    zn[k1] = own ? mine : theirs;
+  }
+  if (!live) return;
+#pragma unroll
+  for (int k1 = 0; k1 < N1 / 2; ++k1) split_put(u[k1], zn[k1], dA + col + N2 * k1, dB + col + N2 * k1);
+  if (t == 0) split_put(u[N1 / 2], u[N1 / 2], dA + N / 2, dB + N / 2);
 }
 
 // Rows inverse, step 1, lane n1: Z_n = A_n + i B_n from the half spectra

@@ -123,11 +123,13 @@ template <typename T> int default_plane_mode(int nx, int ny, int nz);
 // Kernels one forward (or inverse) transform launches: 1 on the plane path, 2 otherwise.
 template <typename T> int transform_launches(const TransformGeom &g);
 
-// Forward: real field [ny][nz][nx] (times in_scale) -> spectrum [ny][nz][nx/2+1],
-// for fields 0 .. g.nb-1.
+// Forward: real field [ny][nz][nx] -> spectrum [ny][nz][nx/2+1], for fields
+// 0 .. g.nb-1.  The FFT modes hand over twice the spectrum and the inverse
+// takes the factor out again (fft2.cuh split_put); the solve in between is
+// linear, and zrhs / zsol carry the true values.
 template <typename T>
 cudaError_t launch_forward(const TransformGeom &g, Ptr3<const T *> in, Ptr3<cplx<T> *> S, const cplx<T> *twx,
-                           const cplx<T> *twz, T in_scale, cudaStream_t st);
+                           const cplx<T> *twz, cudaStream_t st);
 // Inverse: spectrum -> out = addend + scale * field (addend may be NULL or equal out).
 template <typename T>
 cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> out, Ptr3<const T *> addend,
@@ -137,15 +139,14 @@ cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> 
 // the same contracts as launch_forward / launch_inverse.
 bool dft_tc_supported(int nx, int nz);
 cudaError_t dft_tc_upload(int nx, int nz, void **fwd, void **inv, size_t *bytes);
-cudaError_t launch_dft_forward(const TransformGeom &g, Ptr3<const float *> in, Ptr3<float2 *> S, float in_scale,
-                               cudaStream_t st);
+cudaError_t launch_dft_forward(const TransformGeom &g, Ptr3<const float *> in, Ptr3<float2 *> S, cudaStream_t st);
 cudaError_t launch_dft_inverse(const TransformGeom &g, Ptr3<float2 *> S, Ptr3<float *> out,
                                Ptr3<const float *> addend, float scale, cudaStream_t st);
 
 // Split passes: x rows then z columns (forward), z columns then x rows (inverse).
 template <typename T>
 cudaError_t launch_axis_forward(const TransformGeom &g, Ptr3<const T *> in, Ptr3<cplx<T> *> S, const cplx<T> *twx,
-                                const cplx<T> *twz, T in_scale, cudaStream_t st);
+                                const cplx<T> *twz, cudaStream_t st);
 template <typename T>
 cudaError_t launch_axis_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> out, Ptr3<const T *> addend,
                                 const cplx<T> *twx, const cplx<T> *twz, T scale, cudaStream_t st);
@@ -156,7 +157,7 @@ cudaError_t launch_axis_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<
 template <typename T> bool cplane_supported(int nx, int nz, int C);
 template <typename T>
 cudaError_t launch_cplane_forward(const TransformGeom &g, int C, Ptr3<const T *> in, Ptr3<cplx<T> *> S,
-                                  const cplx<T> *twx, const cplx<T> *twz, T in_scale, cudaStream_t st);
+                                  const cplx<T> *twx, const cplx<T> *twz, cudaStream_t st);
 template <typename T>
 cudaError_t launch_cplane_inverse(const TransformGeom &g, int C, Ptr3<cplx<T> *> S, Ptr3<T *> out,
                                   Ptr3<const T *> addend, const cplx<T> *twx, const cplx<T> *twz, T scale,

@@ -227,7 +227,7 @@ static int solve_once(ibm_plan_s *p, const PencilParams &pp, const T *in, T *out
   const int nl = transform_launches<T>(g);
   {
     ProfScope ps(p, IBM_K_FORWARD, st, nl);
-    IBM_CUDA_TRY(launch_forward<T>(gf, ptr3(in), ptr3(S), twx, twz, (T)1, st));
+    IBM_CUDA_TRY(launch_forward<T>(gf, ptr3(in), ptr3(S), twx, twz, st));
   }
   {
     ProfScope ps(p, IBM_K_PENCIL, st);
@@ -375,7 +375,7 @@ static int solve_fields_t(ibm_plan_s *p, double c, int nb, const int *field_bc, 
   const int nl = transform_launches<T>(g);
   {
     ProfScope ps(p, IBM_K_FORWARD, st, nl);
-    IBM_CUDA_TRY(launch_forward<T>(g, in3, S, twx, twz, (T)1, st));
+    IBM_CUDA_TRY(launch_forward<T>(g, in3, S, twx, twz, st));
   }
   {
     ProfScope ps(p, IBM_K_PENCIL, st);

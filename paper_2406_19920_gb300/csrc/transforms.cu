@@ -49,7 +49,7 @@ template <typename T, int NX, int NZ> struct PlaneCfg {
   // threads: enough for the largest of the x step-1, x step-3 and z step-1
   // job counts in one round (z step 3 takes N2z / N1z rounds), <= 1024
   static constexpr int N1Z = TwoStep<NZ>::N1;
-  static constexpr int J3 = N2X / 2 + 1;
+  static constexpr int J3 = N2X / 2;
   static constexpr int JMAX0 = CP * N1X > CP * J3 ? CP * N1X : CP * J3;
   static constexpr int JMAX = JMAX0 > CW * N1Z ? JMAX0 : CW * N1Z;
   static constexpr int THREADS = JMAX >= 1024 ? 1024 : (JMAX + 31) / 32 * 32;
@@ -58,13 +58,13 @@ template <typename T, int NX, int NZ> struct PlaneCfg {
 template <typename T, int NX, int NZ>
 __global__ void __launch_bounds__(PlaneCfg<T, NX, NZ>::THREADS)
 k_plane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__ twx,
-            const cplx<T> *__restrict__ twz, T in_scale, double *zrhs) {
+            const cplx<T> *__restrict__ twz, double *zrhs) {
   const T *__restrict__ in = in_[blockIdx.y];
   cplx<T> *__restrict__ S = S_[blockIdx.y];
   using Cfg = PlaneCfg<T, NX, NZ>;
   constexpr int P = Cfg::P, N1X = Cfg::N1X, XPITCH = Cfg::XPITCH, CP = Cfg::CP, CW = Cfg::CW;
   constexpr int kPlaneThreads_ = Cfg::THREADS;
-  constexpr int N1Z = TwoStep<NZ>::N1, N2Z = TwoStep<NZ>::N2, J3 = Cfg::N2X / 2 + 1;
+  constexpr int N1Z = TwoStep<NZ>::N1, N2Z = TwoStep<NZ>::N2, J3 = Cfg::N2X / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T> *tw2x = reinterpret_cast<cplx<T> *>(smem_raw);
   cplx<T> *tw2z = tw2x + NX;
@@ -81,7 +81,7 @@ k_plane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__
     const int np = min(CP, NZ / 2 - p0);
     for (int job = tid; job < np * N1X; job += kPlaneThreads_) {
       const int p = job / N1X, n1 = job - p * N1X;
-      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, in_scale, n1, tw2x, X + (p * N1X + n1) * XPITCH);
+      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, n1, tw2x, X + (p * N1X + n1) * XPITCH);
     }
     __syncthreads();
     for (int job = tid; job < np * J3; job += kPlaneThreads_) {
@@ -104,7 +104,7 @@ k_plane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__
       const int k2 = job / CW, c = job - k2 * CW;
       if (c < nc) {
         const cplx<T> u0 = col_step3<T, NZ, false, CW>(X, c, k2, dst + c0 + c, P);
-        if (zrhs && c0 + c == 0 && k2 == 0) zrhs[j] = (double)u0.x;
+        if (zrhs && c0 + c == 0 && k2 == 0) zrhs[j] = 0.5 * (double)u0.x;
       }
     }
     __syncthreads();
@@ -135,7 +135,7 @@ k_plane_inv(Ptr3<cplx<T> *> S_, Ptr3<T *> out_, Ptr3<const T *> add_, const cplx
   pdl_wait();  // the fields below are the predecessor's output
   __syncthreads();
   const cplx<T> *src = S + (size_t)j * NZ * P;
-  const cplx<T> z0 = zsol ? mk<T>((T)zsol[j], (T)0) : mk<T>((T)0, (T)0);
+  const cplx<T> z0 = zsol ? mk<T>((T)(2.0 * zsol[j]), (T)0) : mk<T>((T)0, (T)0);
   for (int c0 = 0; c0 < P; c0 += CW) {
     const int nc = min(CW, P - c0);
     for (int job = tid; job < CW * N1Z; job += kPlaneThreads_) {
@@ -189,19 +189,19 @@ template <typename T> static bool plane_supported(int nx, int nz) {
 
 template <typename T>
 cudaError_t launch_forward(const TransformGeom &g, Ptr3<const T *> in, Ptr3<cplx<T> *> S, const cplx<T> *twx,
-                           const cplx<T> *twz, T in_scale, cudaStream_t st) {
+                           const cplx<T> *twz, cudaStream_t st) {
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   if constexpr (sizeof(T) == 4) {
-    if (g.use_plane == kPlaneDft && g.dft_fwd) return launch_dft_forward(g, in, S, in_scale, st);
+    if (g.use_plane == kPlaneDft && g.dft_fwd) return launch_dft_forward(g, in, S, st);
   }
   if (g.use_plane >= 2 && cplane_supported<T>(nx, nz, g.use_plane))
-    return launch_cplane_forward<T>(g, g.use_plane, in, S, twx, twz, in_scale, st);
+    return launch_cplane_forward<T>(g, g.use_plane, in, S, twx, twz, st);
   if (g.use_plane == 1 && plane_supported<T>(nx, nz)) {
 #define X(a, b)                                                                                  \
   if (nx == a && nz == b) {                                                                      \
     if constexpr (PlaneCfg<T, a, b>::ok) {                                                       \
       { cudaError_t e = ensure_max_smem<k_plane_fwd<T, a, b>>(); if (e) return e; }              \
-      IBM_KTRY(launch_pdl(k_plane_fwd<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, in, S, twx, twz, in_scale, g.zrhs)); \
+      IBM_KTRY(launch_pdl(k_plane_fwd<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, in, S, twx, twz, g.zrhs)); \
       return cudaGetLastError();                                                                 \
     }                                                                                            \
   }
@@ -209,7 +209,7 @@ cudaError_t launch_forward(const TransformGeom &g, Ptr3<const T *> in, Ptr3<cplx
 #undef X
   }
   // axis path: x rows then z columns
-  return launch_axis_forward<T>(g, in, S, twx, twz, in_scale, st);
+  return launch_axis_forward<T>(g, in, S, twx, twz, st);
 }
 
 template <typename T>
@@ -226,7 +226,7 @@ cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> 
   if (nx == a && nz == b) {                                                                      \
     if constexpr (PlaneCfg<T, a, b>::ok) {                                                       \
       { cudaError_t e = ensure_max_smem<k_plane_inv<T, a, b>>(); if (e) return e; }              \
-      IBM_KTRY(launch_pdl(k_plane_inv<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, S, out, addend, twx, twz, scale, g.zsol)); \
+      IBM_KTRY(launch_pdl(k_plane_inv<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, S, out, addend, twx, twz, (T)0.5 * scale, g.zsol)); \
       return cudaGetLastError();                                                                 \
     }                                                                                            \
   }
@@ -237,9 +237,9 @@ cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> 
 }
 
 template cudaError_t launch_forward<float>(const TransformGeom &, Ptr3<const float *>, Ptr3<float2 *>, const float2 *,
-                                           const float2 *, float, cudaStream_t);
+                                           const float2 *, cudaStream_t);
 template cudaError_t launch_forward<double>(const TransformGeom &, Ptr3<const double *>, Ptr3<double2 *>,
-                                            const double2 *, const double2 *, double, cudaStream_t);
+                                            const double2 *, const double2 *, cudaStream_t);
 template cudaError_t launch_inverse<float>(const TransformGeom &, Ptr3<float2 *>, Ptr3<float *>, Ptr3<const float *>,
                                            const float2 *, const float2 *, float, cudaStream_t);
 template cudaError_t launch_inverse<double>(const TransformGeom &, Ptr3<double2 *>, Ptr3<double *>,

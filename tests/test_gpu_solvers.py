@@ -357,3 +357,25 @@ def test_invalid_arguments_rejected_before_launch():
             ibm.ibm_helmholtz_solve(plan, -1.0, 0, x, x)
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("prec", [ibm.IBM_FP64, ibm.IBM_FP32_REFINED])
+@pytest.mark.parametrize("n", [8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512])
+def test_split_rows_every_length_last_cta_partial(n, prec, monkeypatch):
+    """x rows and z columns of every length through the split passes (9 planes
+    of 12 or n rows: the row pairs and the columns do not fill the last CTA)."""
+    monkeypatch.setenv("IBM_PLANE_MODE", "0")
+    dt, tol = (torch.float64, TOL_FP64) if prec == ibm.IBM_FP64 else (torch.float32, TOL_FP32)
+    for nx, nz in ((n, 12), (12, n)):
+        g = grid(nx, 9, nz)
+        b = synth.white_noise(nx, 9, nz, workload=15, stream=n).astype(np.float32).astype(np.float64) + 0.25
+        ref, mean_b = O.poisson_solve(b, g)
+        plan = _plan(nx, 9, nz, g, prec)
+        try:
+            rhs = dev(b, dt)
+            phi = torch.empty_like(rhs)
+            info = ibm.ibm_poisson_solve(plan, rhs, phi, info=True)
+            assert rel_err(host(phi), ref) <= tol
+            assert abs(info["removed_mean"] - mean_b) <= (1e-12 if prec == ibm.IBM_FP64 else 1e-6)
+        finally:
+            ibm.ibm_plan_destroy(plan)
