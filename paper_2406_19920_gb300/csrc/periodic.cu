@@ -9,11 +9,16 @@
 //   Poisson    x = -f / lambda, the (0,0,0) mode set to 0 (mean(phi) = 0);
 //   Helmholtz  x =  f / (1 + c lambda).
 // A CTA takes W consecutive pencils (every access a run of W complex
-// values); both y-transforms are the two-step register FFT of fft2.cuh with
-// one shared-memory exchange each, and the divided spectrum crosses shared
-// memory once between them.  For the Poisson solve an extra CTA sums the
-// FP64 plane sums of b (from the forward x/z transform) into the removed
-// mean.
+// values).  With N = N1 N2 the forward transform's step 3 leaves the modes
+// ky = k2 + N2 k1, k1 < N1, in the registers of the thread of k2, and those
+// are one step-1 group of the inverse transform split the other way round
+// (N2 lanes, length-N1 DFTs): the thread divides them by their eigenvalues
+// and runs on into the inverse, whose exchange goes back to the very entries
+// of shared memory the thread read.  Two exchanges and three barriers per
+// pencil in one buffer; bound by the global accesses (512 x 256 x 256 FP32:
+// 104 us a launch with the divide a pass of its own and a second buffer, 61 us
+// now, 4.4 TB/s).  For the Poisson solve an extra CTA sums the FP64 plane sums
+// of b (from the forward x/z transform) into the removed mean.
 #include "fft2.cuh"
 #include "internal.h"
 
@@ -22,12 +27,10 @@ namespace ibm {
 template <typename T, int N> struct YCfg {
   static constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
   static constexpr int WMIN = sizeof(T) == 4 ? 16 : 8, WMAX = 64;
-  static constexpr int WT0 = 256 / N1;
-  static constexpr int WS = (int)(32768 / ((size_t)N * sizeof(cplx<T>)));  // each of X, Y <= 32 KB
-  static constexpr int WT = WT0 < WS ? WT0 : WS;
-  static constexpr int W = WT < WMIN ? WMIN : (WT > WMAX ? WMAX : WT);
+  static constexpr int WT0 = (sizeof(T) == 4 ? 256 : 64) / N1;
+  static constexpr int W = WT0 < WMIN ? WMIN : (WT0 > WMAX ? WMAX : WT0);
   static constexpr int THREADS = W * N1;
-  static constexpr size_t smem = sizeof(cplx<T>) * ((size_t)N + 2 * (size_t)N * W);
+  static constexpr size_t smem = sizeof(cplx<T>) * ((size_t)N + (size_t)N * W) + sizeof(T) * N;
 };
 
 template <typename T, int N>
@@ -38,9 +41,10 @@ k_ypencil(cplx<T> *__restrict__ S, const cplx<T> *__restrict__ tw, const T *__re
   constexpr int N1 = Cfg::N1, N2 = Cfg::N2, W = Cfg::W;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T> *tw2 = reinterpret_cast<cplx<T> *>(smem_raw);
-  cplx<T> *X = tw2 + N;      // [N1][N2][W] exchange of both transforms
-  cplx<T> *Y = X + N * W;    // [N][W] divided y-spectrum
+  cplx<T> *X = tw2 + N;  // [N1][N2][W] exchange of both transforms
+  T *ly = reinterpret_cast<T *>(X + N * W);  // lambda_y
   load_step_twiddles<T, N>(tw2, tw);
+  for (int i = threadIdx.x; i < N; i += blockDim.x) ly[i] = lamy[i];
   pdl_wait();
   if (pp.zero_mode && blockIdx.x == gridDim.x - 1) {
     // removed mean of b: the FP64 sum of the plane sums (zrhs) / (nx ny nz)
@@ -76,32 +80,37 @@ k_ypencil(cplx<T> *__restrict__ S, const cplx<T> *__restrict__ tw, const T *__re
   // forward y-transform, step 1
   if (live) col_step1<T, N, false, W>(base, plane, tid / W, tw2, X + (tid / W) * N2 * W + c, false, mk<T>(0, 0));
   __syncthreads();
-  // step 3 and the divide, into Y in natural ky order
+  // forward step 3, the divide and the inverse's step 1, in the registers of the thread of k2
   if (live) {
     for (int k2 = tid / W; k2 < N2; k2 += N1) {
-      col_step3_at<T, N, false, W>(X, c, k2, [&](int a, int b) {
-        const int ky = a + N2 * b;
-        return Y + ky * W + c;
-      });
+      cplx<T> *x = X + k2 * W + c;  // entries N2 W apart
+      cplx<T> u[N1];
+#pragma unroll
+      for (int n1 = 0; n1 < N1; ++n1) u[n1] = x[n1 * N2 * W];
+      reg_dft<false, N1>(u);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) {
+        const T eig = g_add + g_mul * (lxz + ly[k2 + N2 * k1]);
+        const T s = eig != (T)0 ? sgn * inv_n / eig : (T)0;  // the (0,0,0) Poisson mode -> 0
+        u[k1] = cscale(u[k1], s);
+      }
+      reg_dft<true, N1>(u);
+      x[0] = u[0];
+#pragma unroll
+      for (int m = 1; m < N1; ++m) x[m * N2 * W] = cmulc(u[m], tw2[k2 * N1 + m]);
     }
   }
   __syncthreads();
+  // inverse step 3: rows m + N1 j
   if (live) {
-    for (int ky = tid / W; ky < N; ky += N1) {
-      const T eig = g_add + g_mul * (lxz + lamy[ky]);
-      const cplx<T> f = Y[ky * W + c];
-      const T s = eig != (T)0 ? sgn * inv_n / eig : (T)0;  // the (0,0,0) Poisson mode -> 0
-      Y[ky * W + c] = mk<T>(f.x * s, f.y * s);
-    }
+    const int m = tid / W;
+    cplx<T> u[N2];
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) u[k2] = X[(m * N2 + k2) * W + c];
+    reg_dft<true, N2>(u);
+#pragma unroll
+    for (int j = 0; j < N2; ++j) base[(size_t)(m + N1 * j) * plane] = u[j];
   }
-  __syncthreads();
-  // inverse y-transform
-  if (live)
-    col_step1_at<T, N, true, W>([&](int a, int b) { return Y + (a + N1 * b) * W + c; }, tid / W, tw2,
-                                X + (tid / W) * N2 * W + c, false, mk<T>(0, 0));
-  __syncthreads();
-  if (live)
-    for (int k2 = tid / W; k2 < N2; k2 += N1) col_step3<T, N, true, W>(X, c, k2, base, plane);
 }
 
 #define IBM_Y_N(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512)

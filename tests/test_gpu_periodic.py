@@ -123,3 +123,22 @@ def test_periodic_plan_rejections():
         assert e.value.code == ibm.IBM_ERR_ARG
     finally:
         ibm.ibm_plan_destroy(wall)
+
+
+@pytest.mark.parametrize("ny", [8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512])
+def test_periodic_every_y_length(ny):
+    """Every length of the y transforms (the inverse splits it the other way
+    round); 56 pencils, so the last CTA is partly empty."""
+    shape = (12, ny, 8)
+    b = synth.white_noise(12, ny, 8, workload=82, stream=ny).astype(np.float32).astype(np.float64)
+    for prec, dt, tol in ((ibm.IBM_FP64, torch.float64, TOL_FP64), (ibm.IBM_FP32_REFINED, torch.float32, TOL_FP32)):
+        g, plan = _plan(shape, prec)
+        try:
+            rhs = dev(b, dt)
+            x = torch.empty_like(rhs)
+            ibm.ibm_poisson_solve(plan, rhs, x)
+            assert rel_err(host(x), O.poisson_solve(b, g, ybc=O.PERIODIC)[0]) <= tol
+            ibm.ibm_helmholtz_solve(plan, 0.02, ibm.IBM_FIELD_PERIODIC, rhs, x)
+            assert rel_err(host(x), O.helmholtz_solve(b, g, 0.02, O.PERIODIC)) <= tol
+        finally:
+            ibm.ibm_plan_destroy(plan)
