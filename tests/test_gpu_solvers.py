@@ -379,3 +379,37 @@ def test_split_rows_every_length_last_cta_partial(n, prec, monkeypatch):
             assert abs(info["removed_mean"] - mean_b) <= (1e-12 if prec == ibm.IBM_FP64 else 1e-6)
         finally:
             ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("mode", [2, 3])
+@pytest.mark.parametrize("ny", [8, 9, 17, 33, 64, 129, 511])
+def test_fp64_sweeps_constant_from_the_converged_row(ny, mode, monkeypatch):
+    """The two-ended FP64 sweeps go on with constant pivots once the warp's
+    pencils have converged: at once (small c), within the rows, late or never
+    (Poisson, large c), over the three wall kinds and the smallest halves.
+    Tolerance: TOL_FP64, or kappa eps where that is more (I - c L with
+    eigenvalues up to 1 + c (4/hx^2 + 4/hy^2 + 4/hz^2) and from 1 on, or from
+    1 + c (pi / 2 / Ly)^2 between Dirichlet walls: 1e-11 at 511 rows, c = 50,
+    where the oracle's own rounding is as large)."""
+    monkeypatch.setenv("IBM_PENCIL_MODE", str(mode))
+    g = grid(24, ny, 12)
+    lam_max = sum(4.0 / h ** 2 for h in g[3:])
+    lam_min = (0.5 * math.pi / (ny * g[4])) ** 2
+    b = synth.white_noise(24, ny, 12, workload=16, stream=ny)
+    plan = _plan(24, ny, 12, g, ibm.IBM_FP64)
+    try:
+        rhs = dev(b, torch.float64)
+        x = torch.empty_like(rhs)
+        ibm.ibm_poisson_solve(plan, rhs, x)
+        assert rel_err(host(x), O.poisson_solve(b, g)[0]) <= TOL_FP64
+        for c in (5e-6, 1e-3, 50.0):
+            for bc in (O.NEUMANN, O.CELL_DIRICHLET, O.FACE_DIRICHLET):
+                bb = b.copy()
+                if bc == O.FACE_DIRICHLET:
+                    bb[0] = 0.0
+                ibm.ibm_helmholtz_solve(plan, c, bc, dev(bb, torch.float64), x)
+                kappa = (1 + c * lam_max) / (1 + c * (lam_min if bc != O.NEUMANN else 0.0))
+                tol = max(TOL_FP64, kappa * np.finfo(np.float64).eps)
+                assert rel_err(host(x), O.helmholtz_solve(bb, g, c, bc)) <= tol, (c, bc)
+    finally:
+        ibm.ibm_plan_destroy(plan)
