@@ -151,13 +151,13 @@ int ibm_plan_destroy(ibm_plan plan);
 int ibm_plan_set_delta(ibm_plan plan, int kernel);
 /* Spreading (Eq. 2d) used by ibm_spread / ibm_substep.
  *   IBM_SPREAD_ATOMIC  (default) atomic spreading.  From 40,000 markers on,
- *                      with shared-memory pre-aggregation: a CTA of 256
- *                      (marker, component) entries whose stencils fit a small
- *                      box adds them into shared memory first and then each
- *                      non-zero box point to f with one global atomic; other
- *                      CTAs, and smaller marker sets, add directly as
- *                      IBM_SPREAD_ATOMIC_DIRECT.  The order of the additions,
- *                      and so the last bits of f, vary from run to run.
+ *                      with shared-memory pre-aggregation: a CTA of about 100
+ *                      markers whose stencils fit a small box adds them into
+ *                      shared memory first and then each non-zero box point
+ *                      to f with one global atomic; other CTAs, and smaller
+ *                      marker sets, add to f directly.  The order of the
+ *                      additions, and so the last bits of f, vary from run to
+ *                      run.
  *   IBM_SPREAD_ATOMIC_DIRECT  the paper's L1 kernel (Sec. 2.3.2) as it
  *                      stands: one thread per (marker, component) adds its
  *                      S^3 shares with global atomics.

@@ -15,7 +15,8 @@
 // of an accepted marker is a stored unknown (v's wall face 0 included:
 // accepted markers give it zero weight).
 //
-// One thread per (marker, component).  The stencil origin and offset are
+// One thread per (marker, component), but for FP32 spreading (IBM_SPREAD_ATOMIC),
+// which puts the lanes of a warp on the points of a stencil.  The stencil origin and offset are
 // computed in FP64 on the FP64 path and in float-float on the FP32 path, so
 // that the weights see the marker position without the FP32 rounding of
 // X/h; the weights and sums run in the plan precision.  Spreading
@@ -23,6 +24,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <mutex>
 
 #include "plan.h"
 #include "tma.cuh"
@@ -84,6 +86,39 @@ template <typename T> __device__ __forceinline__ T phi_peskin4(T r) {
   if (a <= (T)1) return ((T)3 - (T)2 * a + sqrt((T)1 + (T)4 * a - (T)4 * a * a)) / (T)8;
   if (a <= (T)2) return ((T)5 - (T)2 * a - sqrt(fmax((T)0, (T)-7 + (T)12 * a - (T)4 * a * a))) / (T)8;
   return (T)0;
+}
+
+// The S weights along one axis from the offset f of the stencil's first point,
+// with the one square root they share.  Three-point kernel: with r = f - 1 in
+// [-1/2, 1/2] and s = sqrt(1 - 3 r^2), phi(r) = (1 + s) / 3 and phi(r +- 1) =
+// (2 -+ 3 r - s) / 6 (the far branch's 1 - 3 (1 - |r +- 1|)^2 is 1 - 3 r^2).
+// Four-point kernel: with r = f - 1 in [0, 1] and s = sqrt(1 + 4 r (1 - r)),
+// phi(r), phi(1 - r) = (3 - 2 r + s) / 8, (1 + 2 r + s) / 8 and phi(1 + r),
+// phi(2 - r) = (3 - 2 r - s) / 8, (1 + 2 r - s) / 8.
+// The thirds are x c + x c' with c' the rounding error of c = 1/3: FP32's 1/3
+// alone would scale every weight by 1 + 3e-8.
+__device__ __forceinline__ float third(float x) {
+  constexpr float c = (float)(1.0 / 3.0);
+  return fmaf(x, c, x * (float)(1.0 / 3.0 - (double)c));
+}
+__device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
+
+template <typename T, int S> __device__ __forceinline__ void delta_weights(T f, T (&w)[S]) {
+  const T r = f - (T)1;
+  if constexpr (S == 3) {
+    const T s = sqrt(fma((T)-3 * r, r, (T)1));
+    const T far = (T)2 - s;
+    w[0] = third((T)0.5 * fma((T)-3, r, far));
+    w[1] = third((T)1 + s);
+    w[2] = third((T)0.5 * fma((T)3, r, far));
+  } else {
+    const T s = sqrt(fma((T)4 * r, (T)1 - r, (T)1));
+    const T lo = fma((T)-2, r, (T)3), hi = fma((T)2, r, (T)1);
+    w[0] = (lo - s) * (T)0.125;
+    w[1] = (lo + s) * (T)0.125;
+    w[2] = (hi + s) * (T)0.125;
+    w[3] = (hi - s) * (T)0.125;
+  }
 }
 
 __device__ __forceinline__ int wrap(int i, int n) {
@@ -167,12 +202,13 @@ k_interp(IbmGrid g, int n, const T *X, const T *__restrict__ u, const T *__restr
   stencil_origin<T, S>(g, c, mx, my, mz, bx, by, bz, fx, fy, fz);
   const T *f = c == 0 ? u : c == 1 ? v : w;
   const T *df = c == 0 ? du : c == 1 ? dv : dw;
-  T wx[S], wz[S];
+  T wx[S], wys[S], wz[S];
+  delta_weights<T, S>(fx, wx);
+  delta_weights<T, S>(fy, wys);
+  delta_weights<T, S>(fz, wz);
   int ix[S], kz[S];
 #pragma unroll
   for (int q = 0; q < S; ++q) {
-    wx[q] = S == 3 ? phi_roma3<T>(fx - (T)q) : phi_peskin4<T>(fx - (T)q);
-    wz[q] = S == 3 ? phi_roma3<T>(fz - (T)q) : phi_peskin4<T>(fz - (T)q);
     ix[q] = wrap(bx + q, g.nx);
     kz[q] = wrap(bz + q, g.nz);
   }
@@ -182,7 +218,7 @@ k_interp(IbmGrid g, int n, const T *X, const T *__restrict__ u, const T *__restr
   for (int qy = 0; qy < S; ++qy) {
     const int j = by + qy;
     if (j < jlo || j > g.ny - 1) continue;
-    const T wy = S == 3 ? phi_roma3<T>(fy - (T)qy) : phi_peskin4<T>(fy - (T)qy);
+    const T wy = wys[qy];
 #pragma unroll
     for (int qz = 0; qz < S; ++qz) {
       const int row = (j * g.nz + kz[qz]) * g.nx;
@@ -217,12 +253,13 @@ k_spread(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, con
   stencil_origin<T, S>(g, c, X[3 * m], X[3 * m + 1], X[3 * m + 2], bx, by, bz, fx, fy, fz);
   T *f = c == 0 ? fu : c == 1 ? fv : fw;
   const T amp = scale * F[t] * dV[m] * (T)g.vol_inv;
-  T wx[S], wz[S];
+  T wx[S], wys[S], wz[S];
+  delta_weights<T, S>(fx, wx);
+  delta_weights<T, S>(fy, wys);
+  delta_weights<T, S>(fz, wz);
   int ix[S], kz[S];
 #pragma unroll
   for (int q = 0; q < S; ++q) {
-    wx[q] = S == 3 ? phi_roma3<T>(fx - (T)q) : phi_peskin4<T>(fx - (T)q);
-    wz[q] = S == 3 ? phi_roma3<T>(fz - (T)q) : phi_peskin4<T>(fz - (T)q);
     ix[q] = wrap(bx + q, g.nx);
     kz[q] = wrap(bz + q, g.nz);
   }
@@ -231,7 +268,7 @@ k_spread(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, con
   for (int qy = 0; qy < S; ++qy) {
     const int j = by + qy;
     if (j < jlo || j > g.ny - 1) continue;
-    const T wy = S == 3 ? phi_roma3<T>(fy - (T)qy) : phi_peskin4<T>(fy - (T)qy);
+    const T wy = wys[qy];
 #pragma unroll
     for (int qz = 0; qz < S; ++qz) {
       const int row = (j * g.nz + kz[qz]) * g.nx;
@@ -239,6 +276,212 @@ k_spread(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, con
 #pragma unroll
       for (int qx = 0; qx < S; ++qx) atomicAdd(f + row + ix[qx], a * wx[qx]);
     }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// FP32 spreading: one warp for kMkWarp markers, its lanes on the points of a
+// stencil.
+//
+// With one thread per (marker, component) the 32 lanes of an atomic fall on 32
+// stencils, and each is a request of its own to L2 (or, in shared memory,
+// collides with the lanes of neighbouring markers).  Here a stencil's S^3
+// points go to the lanes of one instruction (27 of 32, or 64 in two): the S
+// neighbours along x share a request and no two lanes share an address.  The
+// weights and origins of the kMkWarp markers' six axes (x, y, z with and
+// without the half-cell shift; every component uses three of them) are formed
+// at once, a lane per axis, and go through shared memory.  Same products as
+// k_spread, summed in another order.  FP64 keeps one thread per (marker,
+// component): it is bound by FP64 instructions, and a lane per point would
+// repeat them.  Interpolation keeps it too: L1 serves its gathers (100k
+// markers 23 us against 32 with lanes on points).
+// Measured (20k / 39k markers on a sphere at 128^3): 22.9 / 31.6 us with a
+// thread per (marker, component), 10.2 / 14.8 us.
+// ---------------------------------------------------------------------------
+constexpr int kMkWarp = 5, kMkWarps = 4;  // markers a warp, warps a CTA
+
+template <int S> struct MkWeights {
+  float w[kMkWarp][6][4];  // weights of axis c (entry c: no shift, c + 3: half-cell shift)
+  int b[kMkWarp][6];       // stencil origins (WRAP: x, z wrapped into the periodic range)
+  float x[3 * kMkWarp];    // positions
+  float amp[3 * kMkWarp];  // amplitudes
+};
+
+// Loads the nm markers from m0 on and fills m; returns the markers that the
+// wall rule accepts (a mask, the same in every lane; nothing is filled in for
+// the others) and reports the others.
+template <int S, bool WRAP>
+__device__ __forceinline__ unsigned mk_setup(const IbmGrid &g, MkWeights<S> &m, int m0, int nm, int lane,
+                                             const float *X, const float *F, const float *dV, float scale) {
+  if (lane < 3 * nm) {
+    const int t = 3 * m0 + lane;
+    m.x[lane] = X[t];
+    m.amp[lane] = scale * F[t] * dV[m0 + lane / 3] * (float)g.vol_inv;
+  }
+  __syncwarp();
+  bool ok = false;
+  if (lane < nm) {
+    ok = clear_of_walls<S>(g, m.x[3 * lane + 1]);
+    if (!ok) report_wall(g);
+  }
+  const unsigned okm = __ballot_sync(0xffffffffu, ok);
+  const int mk = lane / 6, cb = lane - 6 * mk, ax = cb % 3;
+  if (lane < 6 * kMkWarp && ((okm >> mk) & 1)) {
+    int b;
+    float f, w[S];
+    axis_origin<S>(m.x[3 * mk + ax], 0.0, ax == 0 ? g.ih_hi[0] : ax == 1 ? g.ih_hi[1] : g.ih_hi[2],
+                   ax == 0 ? g.ih_lo[0] : ax == 1 ? g.ih_lo[1] : g.ih_lo[2], cb < 3 ? 0.0 : 0.5, b, f);
+    delta_weights<float, S>(f, w);
+    if (WRAP && ax != 1) b = wrap(b, ax == 0 ? g.nx : g.nz);
+    m.b[mk][cb] = b;
+#pragma unroll
+    for (int q = 0; q < S; ++q) m.w[mk][cb][q] = w[q];
+  }
+  __syncwarp();
+  return okm;
+}
+
+// The lane's point e of component c's stencil of marker mk: its weight and
+// its grid indexes i, j, k, not yet wrapped along x and z.
+template <int S>
+__device__ __forceinline__ float mk_point(const MkWeights<S> &m, int mk, int c, int e, int &i, int &j, int &k) {
+  const int qx = e % S, qz = (e / S) % S, qy = e / (S * S);
+  const int cx = c == 0 ? 0 : 3, cy = c == 1 ? 1 : 4, cz = c == 2 ? 2 : 5;
+  i = m.b[mk][cx] + qx;
+  j = m.b[mk][cy] + qy;
+  k = m.b[mk][cz] + qz;
+  return m.amp[3 * mk + c] * m.w[mk][cy][qy] * m.w[mk][cz][qz] * m.w[mk][cx][qx];
+}
+
+// The accepted markers' stencils straight into the field (origins wrapped).
+template <int S>
+__device__ __forceinline__ void mk_add_global(const IbmGrid &g, const MkWeights<S> &m, unsigned okm, int lane,
+                                              float *fu, float *fv, float *fw) {
+#pragma unroll
+  for (int e0 = 0; e0 < S * S * S; e0 += 32) {
+    const int e = e0 + lane;
+    if (e >= S * S * S) break;
+#pragma unroll
+    for (int mk = 0; mk < kMkWarp; ++mk) {
+      if (!((okm >> mk) & 1)) continue;  // the wall rule: not spread
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float *f = c == 0 ? fu : c == 1 ? fv : fw;
+        int i, j, k;
+        const float a = mk_point<S>(m, mk, c, e, i, j, k);
+        if (i >= g.nx) i -= g.nx;
+        if (k >= g.nz) k -= g.nz;
+        if (j >= (c == 1 ? 1 : 0) && j < g.ny) atomicAdd(f + (j * g.nz + k) * g.nx + i, a);
+      }
+    }
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(32 * kMkWarps)
+k_spread_w(IbmGrid g, int n, const float *__restrict__ X, const float *__restrict__ F,
+           const float *__restrict__ dV, float *fu, float *fv, float *fw, float scale) {
+  __shared__ MkWeights<S> sm[kMkWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int m0 = (blockIdx.x * kMkWarps + warp) * kMkWarp;
+  pdl_wait();
+  if (m0 >= n) return;
+  const unsigned okm = mk_setup<S, true>(g, sm[warp], m0, min(kMkWarp, n - m0), lane, X, F, dV, scale);
+  mk_add_global<S>(g, sm[warp], okm, lane, fu, fv, fw);
+}
+
+// k_spread_box (below) with the lanes on the points: kMkBoxWarps warps of
+// kMkWarp markers add into the CTA's box in shared memory, then its non-zero
+// points go to the field with one global atomic each; boxes too large for the
+// shared budget go to the field directly.  Measured, 100k markers: sphere at
+// 128^3 37.7 us with a thread per (marker, component), 32.2 us; plate at 384 x
+// 256 x 256 with the four-point kernel 82 us, 50 us.  100 markers a CTA (the
+// thread form has 85): with 40 or 80 a CTA more of the sum is left to global
+// FP32 atomics and the dense sphere's error grows (2.2e-7 with 85, 3.0e-7 with
+// 40, 1.9e-7 with 160, which takes 39 us).
+constexpr int kMkBoxWarps = 20;
+constexpr int kMkBoxBytes = 40 * 1024;
+
+template <int S>
+__global__ void __launch_bounds__(32 * kMkBoxWarps)
+k_spread_box_w(IbmGrid g, int n, const float *__restrict__ X, const float *__restrict__ F,
+               const float *__restrict__ dV, float *fu, float *fv, float *fw, float scale) {
+  extern __shared__ __align__(16) unsigned char box_raw[];
+  float *box = reinterpret_cast<float *>(box_raw);
+  MkWeights<S> *sm = reinterpret_cast<MkWeights<S> *>(box_raw + kMkBoxBytes);
+  __shared__ int red[6][kMkBoxWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  MkWeights<S> &m = sm[warp];
+  const int m0 = (blockIdx.x * kMkBoxWarps + warp) * kMkWarp;
+  pdl_wait();
+  const unsigned okm = m0 < n ? mk_setup<S, false>(g, m, m0, min(kMkWarp, n - m0), lane, X, F, dV, scale) : 0u;
+  // bounding box of the CTA's stencil origins (unwrapped)
+  {
+    const int mk = lane / 6, cb = lane - 6 * mk;
+    const bool live = lane < 6 * kMkWarp && ((okm >> mk) & 1);
+    const int b = live ? m.b[mk][cb] : 0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      const bool in = live && cb % 3 == ax;
+      const int mn = __reduce_min_sync(0xffffffffu, in ? b : INT_MAX);
+      const int mx = __reduce_max_sync(0xffffffffu, in ? b : INT_MIN);
+      if (lane == 0) { red[ax][warp] = mn; red[ax + 3][warp] = mx; }
+    }
+  }
+  __syncthreads();
+  int lo[3], dim[3];
+  bool fits = true;
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    int mn = INT_MAX, mx = INT_MIN;
+    for (int w = 0; w < kMkBoxWarps; ++w) { mn = min(mn, red[ax][w]); mx = max(mx, red[ax + 3][w]); }
+    if (mn > mx) return;  // every marker of the CTA was rejected by the wall rule
+    lo[ax] = mn;
+    const long d = (long)mx - mn + S;
+    fits = fits && d <= kMkBoxBytes;
+    dim[ax] = fits ? (int)d : 0;
+  }
+  const long vol_l = (long)dim[0] * dim[1] * dim[2];
+  fits = fits && 3 * vol_l * (long)sizeof(float) <= kMkBoxBytes && dim[0] <= g.nx && dim[2] <= g.nz;
+  if (!fits) {
+    const int mk = lane / 6, cb = lane - 6 * mk, ax = cb % 3;
+    if (lane < 6 * kMkWarp && ((okm >> mk) & 1) && ax != 1) m.b[mk][cb] = wrap(m.b[mk][cb], ax == 0 ? g.nx : g.nz);
+    __syncwarp();
+    mk_add_global<S>(g, m, okm, lane, fu, fv, fw);
+    return;
+  }
+  const int vol = (int)vol_l, nbox = 3 * vol;
+  for (int e = threadIdx.x; e < nbox; e += 32 * kMkBoxWarps) box[e] = 0.f;
+  __syncthreads();
+#pragma unroll
+  for (int e0 = 0; e0 < S * S * S; e0 += 32) {
+    const int e = e0 + lane;
+    if (e >= S * S * S) break;
+#pragma unroll
+    for (int mk = 0; mk < kMkWarp; ++mk) {
+      if (!((okm >> mk) & 1)) continue;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        int i, j, k;
+        const float a = mk_point<S>(m, mk, c, e, i, j, k);
+        atomicAdd(box + c * vol + ((j - lo[1]) * dim[2] + (k - lo[2])) * dim[0] + (i - lo[0]), a);
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nbox; e += 32 * kMkBoxWarps) {
+    const float val = box[e];
+    if (val == 0.f) continue;
+    const int c = e / vol;
+    int r = e - c * vol;
+    const int dy = r / (dim[2] * dim[0]);
+    r -= dy * dim[2] * dim[0];
+    const int dz = r / dim[0], dx = r - dz * dim[0];
+    const int j = lo[1] + dy;
+    if (j < (c == 1 ? 1 : 0) || j > g.ny - 1) continue;
+    const int i = wrap(lo[0] + dx, g.nx), k = wrap(lo[2] + dz, g.nz);
+    float *f = c == 0 ? fu : c == 1 ? fv : fw;
+    atomicAdd(f + ((size_t)j * g.nz + k) * g.nx + i, val);
   }
 }
 
@@ -253,11 +496,14 @@ k_spread(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, con
 // global atomic (x and z wrapped, points beyond the walls dropped as in
 // k_spread).  Otherwise the CTA falls back to k_spread's direct global
 // atomics.  Same sums in another order (FP32 atomics are unordered anyway).
-// Measured on GB300 (FP32, a Fibonacci sphere of radius 0.25 at 128^3): 20k
-// markers 21.2 us against 16.7 us for direct atomics (little contention:
-// the extra phases cost more than they save); 100k markers 38.3 us against
-// 81.6 us.  IBM_SPREAD_ATOMIC therefore takes this kernel from
-// kSpreadBoxMinMarkers markers on.
+// Measured on GB300 (FP32, a Fibonacci sphere of radius 0.25 at 128^3, a
+// thread per (marker, component)): 20k markers 21.2 us against 16.7 us for
+// direct atomics (little contention: the extra phases cost more than they
+// save); 100k markers 38.3 us against 81.6 us.  IBM_SPREAD_ATOMIC therefore
+// pre-aggregates from kSpreadBoxMinMarkers markers on: FP64 in this kernel,
+// FP32 in k_spread_box_w, where direct atomics from the lanes (k_spread_w)
+// would be as fast on sparser sets (100k-marker plate 24 us) but would leave
+// longer FP32 sums to the atomics (dense sphere 6e-7 against 2e-7).
 constexpr int kSpreadBoxMinMarkers = 40000;
 constexpr int kSpreadBoxBytes = 40 * 1024;  // within the default 48 KB limit with the static part
 
@@ -308,12 +554,10 @@ k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F,
   if (!any) return;  // every entry of the CTA was rejected by the wall rule
   const long vol = (long)dim[0] * dim[1] * dim[2];
   const bool use_box = vol > 0 && 3 * vol * (long)sizeof(T) <= kSpreadBoxBytes && dim[0] <= g.nx && dim[2] <= g.nz;
-  T wx[S], wz[S];
-#pragma unroll
-  for (int q = 0; q < S; ++q) {
-    wx[q] = S == 3 ? phi_roma3<T>(fx - (T)q) : phi_peskin4<T>(fx - (T)q);
-    wz[q] = S == 3 ? phi_roma3<T>(fz - (T)q) : phi_peskin4<T>(fz - (T)q);
-  }
+  T wx[S], wys[S], wz[S];
+  delta_weights<T, S>(fx, wx);
+  delta_weights<T, S>(fy, wys);
+  delta_weights<T, S>(fz, wz);
   const int jlo = c == 1 ? 1 : 0;
   if (!use_box) {
     if (!valid) return;
@@ -328,7 +572,7 @@ k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F,
     for (int qy = 0; qy < S; ++qy) {
       const int j = by + qy;
       if (j < jlo || j > g.ny - 1) continue;
-      const T wy = S == 3 ? phi_roma3<T>(fy - (T)qy) : phi_peskin4<T>(fy - (T)qy);
+      const T wy = wys[qy];
 #pragma unroll
       for (int qz = 0; qz < S; ++qz) {
         const int row = (j * g.nz + kz[qz]) * g.nx;
@@ -347,7 +591,7 @@ k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F,
     const int ox = bx - lo[0], oy = by - lo[1], oz = bz - lo[2];
 #pragma unroll
     for (int qy = 0; qy < S; ++qy) {
-      const T wy = S == 3 ? phi_roma3<T>(fy - (T)qy) : phi_peskin4<T>(fy - (T)qy);
+      const T wy = wys[qy];
 #pragma unroll
       for (int qz = 0; qz < S; ++qz) {
         T *rowp = bc + ((oy + qy) * dim[2] + (oz + qz)) * dim[0] + ox;
@@ -751,6 +995,17 @@ static int spread_gather(ibm_plan_s *p, int n, const T *X, const T *F, const T *
   return IBM_OK;
 }
 
+// Raises k_spread_box_w's dynamic shared-memory limit (it has a static part,
+// so not to the per-block maximum), once and thread-safely.
+template <int S> static cudaError_t mk_box_smem(size_t bytes) {
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  std::call_once(once, [&] {
+    err = cudaFuncSetAttribute(k_spread_box_w<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+  return err;
+}
+
 template <typename T>
 cudaError_t launch_spread(const ibm_plan_s *p, int n, const T *X, const T *F, const T *dV, T *fu, T *fv, T *fw,
                           double scale, cudaStream_t st) {
@@ -761,23 +1016,36 @@ cudaError_t launch_spread(const ibm_plan_s *p, int n, const T *X, const T *F, co
     return rc == IBM_OK ? cudaSuccess : cudaErrorMemoryAllocation;
   }
   const IbmGrid g = ibm_grid(p);
-  const int tb = ceil_div(3 * n, 256);
-  if (p->spread == IBM_SPREAD_ATOMIC_DIRECT || n < kSpreadBoxMinMarkers) {
-    if (p->delta == IBM_DELTA_PESKIN4)
-      IBM_KTRY(launch_pdl(k_spread<T, 4>, tb, 256, 0, st, g, n, X, F, dV, fu, fv, fw, (T)scale));
-    else
-      IBM_KTRY(launch_pdl(k_spread<T, 3>, tb, 256, 0, st, g, n, X, F, dV, fu, fv, fw, (T)scale));
-    return cudaGetLastError();
+  if constexpr (sizeof(T) == 4) {
+    if (p->spread == IBM_SPREAD_ATOMIC) {
+      const bool peskin = p->delta == IBM_DELTA_PESKIN4;
+      if (n < kSpreadBoxMinMarkers) {
+        const int wb = ceil_div(n, kMkWarp * kMkWarps);
+        IBM_KTRY(launch_pdl(peskin ? k_spread_w<4> : k_spread_w<3>, wb, 32 * kMkWarps, 0, st, g, n, X, F, dV, fu, fv,
+                            fw, (float)scale));
+      } else {
+        const int wb = ceil_div(n, kMkWarp * kMkBoxWarps);
+        const size_t sb = kMkBoxBytes + kMkBoxWarps * sizeof(MkWeights<3>);  // (MkWeights<4> has the same layout)
+        IBM_KTRY(mk_box_smem<3>(sb));
+        IBM_KTRY(mk_box_smem<4>(sb));
+        IBM_KTRY(launch_pdl(peskin ? k_spread_box_w<4> : k_spread_box_w<3>, wb, 32 * kMkBoxWarps, sb, st, g, n, X, F,
+                            dV, fu, fv, fw, (float)scale));
+      }
+      return cudaGetLastError();
+    }
   }
-  if (p->delta == IBM_DELTA_PESKIN4)
-    IBM_KTRY(launch_pdl(k_spread_box<T, 4>, tb, 256, (size_t)kSpreadBoxBytes, st, g, n, X, F, dV, fu, fv, fw,
-                        (T)scale));
-  else
-    IBM_KTRY(launch_pdl(k_spread_box<T, 3>, tb, 256, (size_t)kSpreadBoxBytes, st, g, n, X, F, dV, fu, fv, fw,
-                        (T)scale));
+  const int tb = ceil_div(3 * n, 256);
+  const bool peskin = p->delta == IBM_DELTA_PESKIN4;
+  if constexpr (sizeof(T) == 8) {
+    if (p->spread == IBM_SPREAD_ATOMIC && n >= kSpreadBoxMinMarkers) {
+      IBM_KTRY(launch_pdl(peskin ? k_spread_box<T, 4> : k_spread_box<T, 3>, tb, 256, (size_t)kSpreadBoxBytes, st, g, n,
+                          X, F, dV, fu, fv, fw, (T)scale));
+      return cudaGetLastError();
+    }
+  }
+  IBM_KTRY(launch_pdl(peskin ? k_spread<T, 4> : k_spread<T, 3>, tb, 256, 0, st, g, n, X, F, dV, fu, fv, fw, (T)scale));
   return cudaGetLastError();
 }
-
 
 template cudaError_t launch_interp<float>(const ibm_plan_s *, int, const float *, const float *, const float *,
                                           const float *, const float *, const float *, const float *, float *,

@@ -304,3 +304,42 @@ def test_box_spread_near_walls_and_unordered(prec):
             assert rel_err(host(got), ref) <= tol
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("kernel", [ibm.IBM_DELTA_ROMA3, ibm.IBM_DELTA_PESKIN4])
+@pytest.mark.parametrize("n", [1, 4, 5, 6, 19, 20, 21, 39999, 40000, 40001])
+def test_fp32_spread_lanes_on_points(n, kernel):
+    """FP32 spreading takes 5 markers a warp, 4 warps a CTA below 40,000 markers
+    and 20 above: last warps and CTAs partly empty, markers across both
+    periodic ends (far outside the box too) and against the walls, every
+    seventh one rejected by the wall rule."""
+    nx, ny, nz = 48, 24, 32
+    g = grid(nx, ny, nz)
+    r = np.random.default_rng(n)
+    half = 1.5 if kernel == ibm.IBM_DELTA_ROMA3 else 2.0
+    X = np.column_stack([0.02 * r.standard_normal(n) + np.where(np.arange(n) % 2, 2 * math.pi, 0.0),
+                         np.where(np.arange(n) % 3, half * g[4] + 1e-3, ny * g[4] - half * g[4] - 1e-3 - 0.01)
+                         + 0.01 * r.random(n),
+                         0.02 * r.standard_normal(n) - np.where(np.arange(n) % 5, 0.0, 4 * math.pi)])
+    X[6::7, 1] = 0.5 * g[4]
+    F, dV = r.standard_normal((n, 3)), 0.5 + r.random(n)
+    X, F, dV = (a.astype(np.float32).astype(np.float64) for a in (X, F, dV))
+    keep = O.clear_of_walls(X, g, kernel)
+    assert (~keep).sum() == len(X[6::7])
+    ref = O.spread(X[keep], F[keep], dV[keep], g, kernel)
+    plan = ibm.ibm_plan_create(nx, ny, nz, g[3:], ibm.IBM_FP32_REFINED, 1)
+    try:
+        ibm.ibm_plan_set_delta(plan, kernel)
+        f = [torch.zeros((ny, nz, nx), dtype=torch.float32, device="cuda") for _ in range(3)]
+        ibm.ibm_spread(plan, n, dev(X, torch.float32), dev(F, torch.float32), dev(dV, torch.float32), *f)
+        if n > 6:
+            with pytest.raises(ibm.IbmError, match="%d marker" % (~keep).sum()):
+                ibm.ibm_plan_check(plan)
+        else:
+            ibm.ibm_plan_check(plan)
+        # tens of thousands of random-signed forces on a few hundred points: a point's FP32 sum over n / 20
+        # markers rounds by about sqrt(n / 20) eps32 of its terms, and the sum itself is sqrt(n / 20) of them
+        for got, want in zip(f, ref):
+            assert rel_err(host(got), want) <= max(TOL_IBM_FP32, math.sqrt(n / 20) * np.finfo(np.float32).eps)
+    finally:
+        ibm.ibm_plan_destroy(plan)
