@@ -18,8 +18,10 @@
 // without printing.  Advection is the conservative MAC form div(u u) with
 // two-point averages (the paper names second-order central differences).
 #include <cmath>
+#include <mutex>
 
 #include "plan.h"
+#include "tma.cuh"
 
 namespace ibm {
 
@@ -53,187 +55,355 @@ template <typename T> struct F3 {
   }
 };
 
-// E1, all three components.  A CTA owns a TX x TZ column tile and marches
-// up JC planes of y; the planes j-1, j, j+1 of u, v, w (and j of p) sit in a
-// shared-memory ring with a one-cell periodic halo in x and z, so every
-// field is read from HBM about once (plus halo and the two extra planes per
-// chunk) and every stencil point comes from shared memory.  Wall rules in
-// y: u, w cell-centred with the no-slip ghost (-value) in the Laplacian and
-// zero wall flux in the advective y-flux; v on faces, zero at the walls
-// (j = 0 stored as the wall, j = ny not stored).
+// E1, all three components.  A CTA owns a TX x TZ column tile (a thread two
+// columns, neighbours in z) and marches up a range of y planes; the planes j
+// and j + 1 of u, v, w and j of p sit in shared memory with a one-cell periodic
+// halo in x and z, copied there asynchronously two planes ahead (16 bytes a
+// copy, the halo columns one by one), and N^{n-2} is loaded a plane ahead, so
+// every field is read from HBM about once.  What a thread needs of plane j - 1 it still holds
+// in registers, and so it does the advective fluxes it formed there: with
+//   XY(i, j) = (u_{j-1} + u_j)(v_{i-1} + v_i),  XZ(i, k) = (u_{k-1} + u_k)(w_{i-1} + w_i),
+//   YZ(j, k) = (v_{k-1} + v_k)(w_{j-1} + w_j)
+// (times 4, on the cell edges) one flux serves the two components it
+// transports, and the y and z neighbours' fluxes are the thread's own but at
+// the ends.  That leaves 82 operations a point (111 with every flux formed
+// where it is used) and 16 shared-memory loads (40).
+// Wall rules in y: u, w cell-centred with the no-slip ghost (-value) in the
+// Laplacian and zero wall flux in the advective y-flux; v on faces, zero at
+// the walls (j = 0 stored as the wall, j = ny not stored).
 //
 // IO: the inflow-outflow walls of Sec. 3 instead.  The y = 0 face carries
 // v = v_lo with u = w = 0 there (the ghost -value and the zero y-flux of
 // u, w are unchanged; v's lower neighbour at j = 1 is v_lo); the y = Ly
 // wall carries the outlet planes uo, wo (u, w at the wall: ghost 2 g - u in
 // the Laplacian, flux v_face * g) and vo (v on the outlet face), [nz][nx].
-constexpr int kExTX = 32, kExTZ = 8, kExJC = 16;
+// Measured (one column a thread, planes j - 1 .. j + 1 in shared memory, 256
+// threads, 16 planes a CTA, against now): FP32 128^3 35.7 -> 23.4 us, 384 x 256
+// x 256 369 -> 240 us (1.31 GB: 5.4 TB/s; bound by instruction issue before, by
+// HBM and the latency of its loads now), FP64 96 x 65 x 64 145 -> 81 us (bound
+// by FP64 operations, 53 us at the pipe's rate, in 24 tiles on 152 SMs).  CTAs of
+// 256 threads: 247 us at 384 x 256 x 256, one plane ahead 277 us.
+constexpr int kExTX = 32, kExTY = 4, kExTZ = 2 * kExTY, kExThreads = kExTX * kExTY;
+
+template <typename T> struct ExTile {
+  static constexpr int VEC = 16 / (int)sizeof(T);     // elements of a 16-byte copy
+  static constexpr int PITCH = kExTX + 2 * VEC;       // a row: VEC (the last is the left halo), TX, VEC
+  static constexpr int ROWS = kExTZ + 2;
+  static constexpr int PL = ROWS * PITCH;
+  static constexpr int CPR = kExTX / VEC;             // 16-byte copies a row
+  static constexpr int OPS = ROWS * (CPR + 2);        // copies a plane (and field)
+  static constexpr int NQ = (OPS + kExThreads - 1) / kExThreads;
+  static constexpr size_t bytes = sizeof(T) * (size_t)PL * 15;  // 4 planes of u, v, w, 3 of p
+};
+
+// Coefficients with the constant factors folded in: dt (a + b) nu / h^2 (vx,
+// vy, vz), dt (a + b) / h (px, py, pz), 1 / (4 h) (qx, qy, qz), dt gamma, dt zeta.
+template <typename T> struct ExCoef {
+  T vx, vy, vz, px, py, pz, qx, qy, qz, gam, zet;
+};
 
 template <typename T, bool IO>
-__global__ void __launch_bounds__(kExTX * kExTZ)
-k_explicit(Geo g, const T *__restrict__ u_, const T *__restrict__ v_, const T *__restrict__ w_,
-           const T *__restrict__ p_, T *Nu, T *Nv, T *Nw, T *__restrict__ du, T *__restrict__ dv,
-           T *__restrict__ dw, T c_visc, T c_pres, T gam, T zet, T dt, T v_lo, const T *__restrict__ uo,
+__global__ void __launch_bounds__(kExThreads, sizeof(T) == 4 ? 4 : 2)
+k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__restrict__ v_,
+           const T *__restrict__ w_, const T *__restrict__ p_, T *Nu, T *Nv, T *Nw, T *__restrict__ du,
+           T *__restrict__ dv, T *__restrict__ dw, ExCoef<T> cf, T v_lo, const T *__restrict__ uo,
            const T *__restrict__ vo, const T *__restrict__ wo) {
+  using Cfg = ExTile<T>;
+  constexpr int VEC = Cfg::VEC, PI = Cfg::PITCH, PL = Cfg::PL, CPR = Cfg::CPR, NQ = Cfg::NQ;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T *su = reinterpret_cast<T *>(smem_raw), *sv = su + 4 * PL, *sw = sv + 4 * PL, *sp = sw + 4 * PL;
+  const int tx = threadIdx.x % kExTX, ty = threadIdx.x / kExTX;
+  const int i0 = blockIdx.x * kExTX, k0 = blockIdx.y * kExTZ;
+  const int jb = blockIdx.z * jc, je = min(ny, jb + jc);
+  const size_t plane = (size_t)nz * nx;
+  // this thread's copies of a plane: source offset, destination, 16 bytes or one element
+  int src[NQ], dst[NQ];
+  bool wide[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int op = threadIdx.x + q * kExThreads;
+    const int r = op < Cfg::OPS ? op / (CPR + 2) : 0, e = op - r * (CPR + 2);
+    const int kk = (k0 - 1 + r + nz) % nz;
+    const int last = min(kExTX, nx - i0);  // the right halo follows the last column of the tile
+    wide[q] = e < CPR;
+    const int x = e < CPR ? i0 + e * VEC : e == CPR ? i0 - 1 + (i0 == 0 ? nx : 0) : (i0 + last == nx ? 0 : i0 + last);
+    src[q] = (op < Cfg::OPS && (e >= CPR || x < nx)) ? kk * nx + x : -1;
+    dst[q] = r * PI + (e < CPR ? VEC + e * VEC : e == CPR ? VEC - 1 : VEC + last);
+  }
+  auto copy = [&](const T *F, int jj, T *buf) {
+    const T *f = F + (size_t)jj * plane;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      if (src[q] < 0) continue;
+      if (wide[q]) cp_async16(buf + dst[q], f + src[q]);
+      else if constexpr (sizeof(T) == 8) cp_async8(buf + dst[q], f + src[q]);
+      else cp_async4(buf + dst[q], f + src[q]);
+    }
+  };
+  // slots of planes j, j + 1 and of the two planes in flight (rotated each plane)
+  int s0 = 0, s1 = PL, s2 = 2 * PL, s3 = 3 * PL;
   pdl_wait();
-  constexpr int TX = kExTX, TZ = kExTZ, HX = TX + 2, HZ = TZ + 2, PL = HX * HZ, NT = TX * TZ;
-  constexpr int NL = (PL + NT - 1) / NT;  // plane elements each thread loads
-  __shared__ T su[3 * PL], sv[3 * PL], sw[3 * PL], sp[2 * PL];
-  const int nx = g.nx, ny = g.ny, nz = g.nz;
-  const int tx = threadIdx.x, tz = threadIdx.y, tid = tz * TX + tx;
-  const int i0 = blockIdx.x * TX, k0 = blockIdx.y * TZ;
-  const int jb = blockIdx.z * kExJC, je = min(ny, jb + kExJC);
-  const int plane = nz * nx;  // < 2^31 for every supported grid
-  // halo-tile element -> offset inside a plane (periodic x, z), fixed for all planes
-  int off[NL];
+  copy(u_, jb, su + s0); copy(v_, jb, sv + s0); copy(w_, jb, sw + s0); copy(p_, jb, sp);
+  if (jb + 1 < ny) { copy(u_, jb + 1, su + s1); copy(v_, jb + 1, sv + s1); copy(w_, jb + 1, sw + s1); }
+  const int i = i0 + tx, k = k0 + 2 * ty;
+  const bool inside = i < nx && k < nz;  // nz is even: both columns or none
+  const int c = (2 * ty + 1) * PI + VEC + tx;  // column 0 in a tile plane; column 1 is c + PI
+  const size_t col = inside ? (size_t)k * nx + i : 0;
+  const T v_wall = IO ? v_lo : (T)0;
+  // of plane j - 1: u (and at i + 1), v, w (and at k + 2), p
+  T ud[2] = {}, uEd[2] = {}, vd[2] = {}, wd[3] = {}, pd[2] = {};
+  if (inside && jb > 0) {
+    const size_t below = (size_t)(jb - 1) * plane;
+    const T *pu = u_ + below, *pv = v_ + below, *pw = w_ + below, *pp = p_ + below;
+    const size_t ce = i + 1 < nx ? col + 1 : col + 1 - nx;
+    const size_t cn = k + 2 < nz ? col + 2 * (size_t)nx : (size_t)i;
 #pragma unroll
-  for (int q = 0; q < NL; ++q) {
-    const int e = tid + q * NT;
-    const int hz = e / HX, hx = e - hz * HX;
-    const int kk = ((k0 - 1 + hz) % nz + nz) % nz, ii = ((i0 - 1 + hx) % nx + nx) % nx;
-    off[q] = e < PL ? kk * nx + ii : -1;
+    for (int z = 0; z < 2; ++z) {
+      ud[z] = pu[col + (size_t)z * nx];
+      uEd[z] = pu[ce + (size_t)z * nx];
+      vd[z] = jb == 1 ? v_wall : pv[col + (size_t)z * nx];
+      wd[z] = pw[col + (size_t)z * nx];
+      pd[z] = pp[col + (size_t)z * nx];
+    }
+    wd[2] = pw[cn];
   }
-  // a plane's tile elements of this thread: fetched into registers one
-  // iteration ahead, stored into the ring after the iteration's compute
-  auto fetch = [&](const T *F, int jj, T (&r)[NL]) {
-    const bool ok = jj >= 0 && jj < ny;
-    const T *src = F + (size_t)(ok ? jj : 0) * plane;
-#pragma unroll
-    for (int q = 0; q < NL; ++q) r[q] = (ok && off[q] >= 0) ? src[off[q]] : (T)0;
-  };
-  auto put = [&](const T (&r)[NL], T *buf) {
-#pragma unroll
-    for (int q = 0; q < NL; ++q)
-      if (off[q] >= 0) buf[tid + q * NT] = r[q];
-  };
-  // ring slots of the planes j-1, j, j+1 (rotated each plane, no modulo)
-  int sm = 0, s0 = PL, sp1 = 2 * PL;
-  {
-    T r[NL];
-    fetch(u_, jb - 1, r); put(r, su + sm);
-    fetch(v_, jb - 1, r); put(r, sv + sm);
-    fetch(w_, jb - 1, r); put(r, sw + sm);
-    fetch(u_, jb, r); put(r, su + s0);
-    fetch(v_, jb, r); put(r, sv + s0);
-    fetch(w_, jb, r); put(r, sw + s0);
-    fetch(u_, jb + 1, r); put(r, su + sp1);
-    fetch(v_, jb + 1, r); put(r, sv + sp1);
-    fetch(w_, jb + 1, r); put(r, sw + sp1);
-    fetch(p_, jb, r); put(r, sp);
-  }
+  cp_async_commit();
+  if (jb + 2 < ny && jb + 1 < je) { copy(u_, jb + 2, su + s2); copy(v_, jb + 2, sv + s2); copy(w_, jb + 2, sw + s2); }
+  if (jb + 1 < je) copy(p_, jb + 1, sp + PL);
+  cp_async_commit();
+  cp_async_wait_group<1>();
   __syncthreads();
-  const int i = i0 + tx, k = k0 + tz;
-  const bool inside = i < nx && k < nz;
-  const int c = (tz + 1) * HX + (tx + 1);  // this column in a halo tile
-  const int col = k * nx + i;
-  T p_prev = (inside && jb > 0) ? p_[(size_t)(jb - 1) * plane + col] : (T)0;
-  const T ihx = (T)g.ihx, ihy = (T)g.ihy, ihz = (T)g.ihz;
-  const T ihx2 = ihx * ihx, ihy2 = ihy * ihy, ihz2 = ihz * ihz;
-  // Every advective flux is a product of two two-point averages,
-  // (a + b)/2 * (c + d)/2: the exact factor 1/4 is carried by the inverse
-  // spacings it is multiplied with (q* = ih* / 4), which leaves each term's
-  // rounding unchanged.
-  const T qx = ihx * (T)0.25, qy = ihy * (T)0.25, qz = ihz * (T)0.25;
-  const bool n_prev = zet != (T)0;  // N^{n-2} unused (and maybe unset) at stage 1
-  int pb = 0;                       // P ring slot of plane j (0 or PL)
-  for (int j = jb; j < je; ++j) {
-    T ru[NL], rv[NL], rw[NL], rp[NL];
-    const bool more = j + 1 < je;
-    if (more) {
-      fetch(u_, j + 2, ru);
-      fetch(v_, j + 2, rv);
-      fetch(w_, j + 2, rw);
-      fetch(p_, j + 1, rp);
-    }
-    if (inside) {
-      const T *Um = su + sm + c, *Uc = su + s0 + c, *Up = su + sp1 + c;
-      const T *Vc = sv + s0 + c, *Vm = sv + sm + c, *Vp = sv + sp1 + c;
-      const T *Wm = sw + sm + c, *Wc = sw + s0 + c, *Wp = sw + sp1 + c;
-      const T *Pc = sp + pb + c;
-      const bool lo = j == 0, hi = j + 1 >= ny;
-      const size_t idx = (size_t)j * plane + col;
-      // tile neighbours: B[dk * HX + di] relative to this column
-      const T p0 = Pc[0];
-      const T u0 = Uc[0], v0 = Vc[0], w0 = Wc[0];
-      // outlet wall values at this column (IO, top row only)
-      T ug = 0, wg = 0, vgo = 0, vgw = 0, vgs = 0;
-      if (IO && hi) {
-        const int iw = i == 0 ? nx - 1 : i - 1, ks = k == 0 ? nz - 1 : k - 1;
-        ug = uo[col]; wg = wo[col]; vgo = vo[col];
-        vgw = vo[k * nx + iw]; vgs = vo[ks * nx + i];
-      }
-      // ---------------- u (x-faces) ----------------
-      {
-        const T ue = Uc[1], uw = Uc[-1], un = Uc[HX], us = Uc[-HX];
-        const T uup = Up[0], udn = Um[0];
-        const T uu = hi ? (IO ? 2 * ug - u0 : -u0) : uup, ud = lo ? -u0 : udn;
-        const T lap = (ue - 2 * u0 + uw) * ihx2 + (un - 2 * u0 + us) * ihz2 + (uu - 2 * u0 + ud) * ihy2;
-        const T uc = u0 + ue, ucm = uw + u0;  // twice the averages
-        const T txx = (uc * uc - ucm * ucm) * qx;
-        // y-flux at the faces j (zero at the wall j = 0) and j+1 (zero at j+1 = ny), times 4
-        const T fy0 = lo ? (T)0 : (Vc[-1] + v0) * (udn + u0);
-        const T fy1 = hi ? (IO ? (vgw + vgo) * (ug + ug) : (T)0) : (Vp[-1] + Vp[0]) * (u0 + uup);
-        const T fz0 = (Wc[-1] + w0) * (us + u0);
-        const T fz1 = (Wc[HX - 1] + Wc[HX]) * (u0 + un);
-        const T N = txx + (fy1 - fy0) * qy + (fz1 - fz0) * qz;
-        const T G = (p0 - Pc[-1]) * ihx;
-        const T np = n_prev ? Nu[idx] : (T)0;
-        du[idx] = dt * (c_visc * lap - c_pres * G - gam * N - zet * np);
-        Nu[idx] = N;
-      }
-      // ---------------- w (z-faces) ----------------
-      {
-        const T we = Wc[1], ww = Wc[-1], wn = Wc[HX], ws = Wc[-HX];
-        const T wup = Wp[0], wdn = Wm[0];
-        const T wu = hi ? (IO ? 2 * wg - w0 : -w0) : wup, wd = lo ? -w0 : wdn;
-        const T lap = (we - 2 * w0 + ww) * ihx2 + (wn - 2 * w0 + ws) * ihz2 + (wu - 2 * w0 + wd) * ihy2;
-        const T wc = w0 + wn, wcm = ws + w0;
-        const T tzz = (wc * wc - wcm * wcm) * qz;
-        const T fx0 = (Uc[-HX] + u0) * (ww + w0);
-        const T fx1 = (Uc[1 - HX] + Uc[1]) * (w0 + we);
-        const T fy0 = lo ? (T)0 : (Vc[-HX] + v0) * (wdn + w0);
-        const T fy1 = hi ? (IO ? (vgs + vgo) * (wg + wg) : (T)0) : (Vp[-HX] + Vp[0]) * (w0 + wup);
-        const T N = tzz + (fx1 - fx0) * qx + (fy1 - fy0) * qy;
-        const T G = (p0 - Pc[-HX]) * ihz;
-        const T np = n_prev ? Nw[idx] : (T)0;
-        dw[idx] = dt * (c_visc * lap - c_pres * G - gam * N - zet * np);
-        Nw[idx] = N;
-      }
-      // ---------------- v (y-faces, interior j = 1..ny-1) ----------------
-      if (lo) {
-        dv[idx] = (T)0;
-        Nv[idx] = (T)0;
-      } else {
-        const T ve = Vc[1], vw = Vc[-1], vn = Vc[HX], vs = Vc[-HX];
-        const T vu = hi ? (IO ? vgo : (T)0) : Vp[0], vd = j - 1 <= 0 ? (IO ? v_lo : (T)0) : Vm[0];
-        const T lap = (ve - 2 * v0 + vw) * ihx2 + (vn - 2 * v0 + vs) * ihz2 + (vu - 2 * v0 + vd) * ihy2;
-        const T vc = v0 + vu, vcm = vd + v0;
-        const T tyy = (vc * vc - vcm * vcm) * qy;
-        const T fx0 = (Um[0] + u0) * (vw + v0);
-        const T fx1 = (Um[1] + Uc[1]) * (v0 + ve);
-        const T fz0 = (Wm[0] + w0) * (vs + v0);
-        const T fz1 = (Wm[HX] + Wc[HX]) * (v0 + vn);
-        const T N = tyy + (fx1 - fx0) * qx + (fz1 - fz0) * qz;
-        const T G = (p0 - p_prev) * ihy;
-        const T np = n_prev ? Nv[idx] : (T)0;
-        dv[idx] = dt * (c_visc * lap - c_pres * G - gam * N - zet * np);
-        Nv[idx] = N;
-      }
-      p_prev = p0;
-    }
-    __syncthreads();
-    if (more) {
-      // plane j+2 replaces plane j-1; the ring rotates
-      put(ru, su + sm);
-      put(rv, sv + sm);
-      put(rw, sw + sm);
-      put(rp, sp + (PL - pb));
-      const int t = sm;
-      sm = s0; s0 = sp1; sp1 = t;
-      pb = PL - pb;
-      __syncthreads();
-    }
+  // of plane j, from the step before: u, u at i + 1, v at k - 1 .. k + 2, v at i -+ 1, w at k .. k + 2
+  T u0[2], uE[2], vc[4], vW[2], vE[2], w0[3];
+  const T *U = su + s0 + c, *V = sv + s0 + c, *W = sw + s0 + c;
+#pragma unroll
+  for (int z = 0; z < 2; ++z) {
+    u0[z] = U[z * PI];
+    uE[z] = U[z * PI + 1];
+    vW[z] = V[z * PI - 1];
+    vE[z] = V[z * PI + 1];
   }
+#pragma unroll
+  for (int z = 0; z < 4; ++z) vc[z] = V[(z - 1) * PI];
+#pragma unroll
+  for (int z = 0; z < 3; ++z) w0[z] = W[z * PI];
+  // fluxes on the lower edges of plane j (zero at the wall j = 0)
+  T xy[2] = {}, xyE[2] = {}, yz[3] = {}, yy[2] = {};
+  if (jb > 0) {
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      xy[z] = (vW[z] + vc[z + 1]) * (ud[z] + u0[z]);
+      xyE[z] = (vc[z + 1] + vE[z]) * (uEd[z] + uE[z]);
+      const T a = vd[z] + vc[z + 1];
+      yy[z] = a * a;
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z) yz[z] = (vc[z] + vc[z + 1]) * (wd[z] + w0[z]);
+  }
+  const bool n_prev = cf.zet != (T)0;  // N^{n-2} unused (and maybe unset) at stage 1
+  int ps = 0;                          // p slot of plane j
+  size_t at = (size_t)jb * plane + col;
+  T nuN[2] = {}, nvN[2] = {}, nwN[2] = {};
+  auto fetch_n = [&](size_t o) {
+    if (n_prev && inside) {
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        nuN[z] = Nu[o + (size_t)z * nx];
+        nvN[z] = Nv[o + (size_t)z * nx];
+        nwN[z] = Nw[o + (size_t)z * nx];
+      }
+    }
+  };
+  fetch_n(at);
+  for (int j = jb; j < je; ++j, at += plane) {
+    if (j > jb) {
+      cp_async_wait_group<1>();
+      __syncthreads();  // planes j + 1 of u, v, w and j of p have landed; plane j - 1's slots are free
+    }
+    const bool lo = j == 0, hi = j + 1 >= ny;
+    if (j + 2 < je) {
+      copy(p_, j + 2, sp + (ps == 0 ? 2 * PL : ps - PL));
+      if (j + 3 < ny) { copy(u_, j + 3, su + s3); copy(v_, j + 3, sv + s3); copy(w_, j + 3, sw + s3); }
+    }
+    cp_async_commit();
+    // N^{n-2} of this plane arrived during the last one
+    T nu[2], nv[2], nw[2];
+#pragma unroll
+    for (int z = 0; z < 2; ++z) { nu[z] = nuN[z]; nv[z] = nvN[z]; nw[z] = nwN[z]; }
+    if (j + 1 < je) fetch_n(at + plane);
+    // plane j + 1 and the fluxes on the upper edges
+    T u1[2], uE1[2], vc1[4], vW1[2], vE1[2], w1[3], xy1[2], xyE1[2], yz1[3], yy1[2], uu[2], wu[2], vu[2];
+    if (!hi) {
+      const T *U1 = su + s1 + c, *V1 = sv + s1 + c, *W1 = sw + s1 + c;
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        u1[z] = U1[z * PI];
+        uE1[z] = U1[z * PI + 1];
+        vW1[z] = V1[z * PI - 1];
+        vE1[z] = V1[z * PI + 1];
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) vc1[z] = V1[(z - 1) * PI];
+#pragma unroll
+      for (int z = 0; z < 3; ++z) w1[z] = W1[z * PI];
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        xy1[z] = (vW1[z] + vc1[z + 1]) * (u0[z] + u1[z]);
+        xyE1[z] = (vc1[z + 1] + vE1[z]) * (uE[z] + uE1[z]);
+        uu[z] = u1[z];
+        wu[z] = w1[z];
+        vu[z] = vc1[z + 1];
+      }
+#pragma unroll
+      for (int z = 0; z < 3; ++z) yz1[z] = (vc1[z] + vc1[z + 1]) * (w0[z] + w1[z]);
+    } else {
+      // the wall above: no plane, no flux; IO: the outlet's values
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        u1[z] = uE1[z] = vW1[z] = vE1[z] = xy1[z] = xyE1[z] = (T)0;
+        uu[z] = -u0[z];
+        wu[z] = -w0[z];
+        vu[z] = (T)0;
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) vc1[z] = (T)0;
+#pragma unroll
+      for (int z = 0; z < 3; ++z) w1[z] = yz1[z] = (T)0;
+      if (IO && inside) {
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+          const int kz = k + z, iw = i == 0 ? nx - 1 : i - 1, ks = kz == 0 ? nz - 1 : kz - 1;
+          const T ug = uo[kz * nx + i], wg = wo[kz * nx + i], vg = vo[kz * nx + i];
+          uu[z] = 2 * ug - u0[z];
+          wu[z] = 2 * wg - w0[z];
+          vu[z] = vg;
+          xy1[z] = (vo[kz * nx + iw] + vg) * (ug + ug);
+          yz1[z] = (vo[ks * nx + i] + vg) * (wg + wg);
+        }
+      }
+    }
+    const T vb[2] = {lo ? v_wall : vc[1], lo ? v_wall : vc[2]};
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const T a = vb[z] + vu[z];
+      yy1[z] = a * a;
+    }
+    // the rest of plane j
+    U = su + s0 + c; V = sv + s0 + c; W = sw + s0 + c;
+    const T *Pp = sp + ps + c;
+    const T uS = U[-PI], uN = U[2 * PI], uES = U[1 - PI], wS = W[-PI];
+    const T uk[4] = {uS, u0[0], u0[1], uN};     // u at k - 1 .. k + 2
+    const T wk[4] = {wS, w0[0], w0[1], w0[2]};  // w at k - 1 .. k + 2
+    const T uEk[3] = {uES, uE[0], uE[1]};       // u at i + 1, k - 1 .. k + 1
+    const T pS = Pp[-PI];
+    T wW[3], xz[3], zz[3], p0[2];
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+      wW[z] = W[z * PI - 1];
+      xz[z] = (wW[z] + w0[z]) * (uk[z] + uk[z + 1]);
+      const T a = wk[z] + wk[z + 1];
+      zz[z] = a * a;
+    }
+#pragma unroll
+    for (int z = 0; z < 2; ++z) p0[z] = Pp[z * PI];
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const size_t o = at + (size_t)z * nx;
+      const T uw = U[z * PI - 1], wE = W[z * PI + 1];
+      // u (x-faces)
+      {
+        const T a = u0[z] + uE[z], b = uw + u0[z];  // twice the averages
+        const T N = (a * a - b * b) * cf.qx + (xy1[z] - xy[z]) * cf.qy + (xz[z + 1] - xz[z]) * cf.qz;
+        const T lx = uE[z] - 2 * u0[z] + uw, lz = uk[z + 2] - 2 * u0[z] + uk[z];
+        const T ly = uu[z] - 2 * u0[z] + (lo ? -u0[z] : ud[z]);
+        if (inside) {
+          du[o] = lx * cf.vx + lz * cf.vz + ly * cf.vy - (p0[z] - Pp[z * PI - 1]) * cf.px - cf.gam * N - cf.zet * nu[z];
+          Nu[o] = N;
+        }
+      }
+      // w (z-faces)
+      {
+        const T xzE = (w0[z] + wE) * (uEk[z] + uEk[z + 1]);
+        const T N = (zz[z + 1] - zz[z]) * cf.qz + (xzE - xz[z]) * cf.qx + (yz1[z] - yz[z]) * cf.qy;
+        const T lx = wE - 2 * w0[z] + wW[z], lz = wk[z + 2] - 2 * w0[z] + wk[z];
+        const T ly = wu[z] - 2 * w0[z] + (lo ? -w0[z] : wd[z]);
+        if (inside) {
+          dw[o] = lx * cf.vx + lz * cf.vz + ly * cf.vy - (p0[z] - (z == 0 ? pS : p0[0])) * cf.pz - cf.gam * N -
+                  cf.zet * nw[z];
+          Nw[o] = N;
+        }
+      }
+      // v (y-faces, interior j = 1 .. ny - 1)
+      {
+        const T v0 = vc[z + 1];
+        const T N = (yy1[z] - yy[z]) * cf.qy + (xyE[z] - xy[z]) * cf.qx + (yz[z + 1] - yz[z]) * cf.qz;
+        const T lx = vE[z] - 2 * v0 + vW[z], lz = vc[z + 2] - 2 * v0 + vc[z];
+        const T ly = vu[z] - 2 * v0 + vd[z];
+        if (inside) {
+          dv[o] = lo ? (T)0
+                     : lx * cf.vx + lz * cf.vz + ly * cf.vy - (p0[z] - pd[z]) * cf.py - cf.gam * N - cf.zet * nv[z];
+          Nv[o] = lo ? (T)0 : N;
+        }
+      }
+    }
+    // plane j becomes plane j - 1
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      ud[z] = u0[z]; u0[z] = u1[z]; uE[z] = uE1[z];
+      vd[z] = vb[z]; vW[z] = vW1[z]; vE[z] = vE1[z];
+      xy[z] = xy1[z]; xyE[z] = xyE1[z]; yy[z] = yy1[z];
+      pd[z] = p0[z];
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) vc[z] = vc1[z];
+#pragma unroll
+    for (int z = 0; z < 3; ++z) { wd[z] = w0[z]; w0[z] = w1[z]; yz[z] = yz1[z]; }
+    const int t = s0;
+    s0 = s1; s1 = s2; s2 = s3; s3 = t;
+    ps = ps == 2 * PL ? 0 : ps + PL;
+  }
+}
+
+// Planes a CTA marches: the split of ny whose CTAs take the fewest rounds of
+// plane steps, a CTA's start counted as two (its first planes are read with
+// nothing to compute).  per_sm: resident CTAs that add to each other's speed
+// (FP32, waiting on memory: all 4; FP64, bound by the SM's FP64 pipe: 1; at
+// 128^3 FP32 a split for 1 takes 33 us and for 4 23 us).
+static int explicit_planes(int nx, int ny, int nz, int per_sm) {
+  static std::once_flag once;
+  static int sms = 0;
+  std::call_once(once, [] {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  });
+  const long tiles = (long)ceil_div(nx, kExTX) * ceil_div(nz, kExTZ);
+  long best = 0;
+  int jc = ny;
+  for (int n = 1; n <= ny; ++n) {  // n chunks
+    const int c = ceil_div(ny, n);
+    if (c < 4 && n > 1) break;
+    const long slots = (long)sms * per_sm;
+    const long cost = ((tiles * ceil_div(ny, c) + slots - 1) / slots) * (c + 2);
+    if (n == 1 || cost < best) { best = cost; jc = c; }
+  }
+  return jc;
+}
+
+template <typename T, bool IO>
+static cudaError_t launch_explicit(const Geo &g, const T *u, const T *v, const T *w, const T *p, T *Nu, T *Nv, T *Nw,
+                                   T *du, T *dv, T *dw, double visc, double pres, double gam, double zet, double dt,
+                                   T v_lo, const T *uo, const T *vo, const T *wo, cudaStream_t st) {
+  ExCoef<T> cf;
+  cf.vx = (T)(dt * visc * g.ihx * g.ihx); cf.vy = (T)(dt * visc * g.ihy * g.ihy); cf.vz = (T)(dt * visc * g.ihz * g.ihz);
+  cf.px = (T)(dt * pres * g.ihx); cf.py = (T)(dt * pres * g.ihy); cf.pz = (T)(dt * pres * g.ihz);
+  cf.qx = (T)(0.25 * g.ihx); cf.qy = (T)(0.25 * g.ihy); cf.qz = (T)(0.25 * g.ihz);
+  cf.gam = (T)(dt * gam); cf.zet = (T)(dt * zet);
+  IBM_KTRY((ensure_max_smem<k_explicit<T, IO>>()));
+  const int jc = explicit_planes(g.nx, g.ny, g.nz, sizeof(T) == 4 ? 4 : 1);
+  const dim3 grid(ceil_div(g.nx, kExTX), ceil_div(g.nz, kExTZ), ceil_div(g.ny, jc));
+  return launch_pdl(k_explicit<T, IO>, grid, dim3(kExThreads), ExTile<T>::bytes, st, g.nx, g.ny, g.nz, jc, u, v, w, p,
+                    Nu, Nv, Nw, du, dv, dw, cf, v_lo, uo, vo, wo);
 }
 
 __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v) {
@@ -552,15 +722,12 @@ static int substep_t(ibm_plan_s *p, ibm_state *s, const ibm_inout *io, int stage
   // E1
   {
     ProfScope ps(p, IBM_K_EXPLICIT, st);
-    const dim3 eg(ceil_div(p->nx, kExTX), ceil_div(p->nz, kExTZ), ceil_div(p->ny, kExJC));
     if (io)
-      IBM_CUDA_TRY(launch_pdl(k_explicit<T, true>, eg, dim3(kExTX, kExTZ), 0, st, g, u, v, w, pr, (T *)s->Nu,
-                              (T *)s->Nv, (T *)s->Nw, du, dv, dw, (T)(ab * nu), (T)ab, (T)gm, (T)zt, (T)dt, v_lo,
-                              (const T *)uo, (const T *)vo, (const T *)wo));
+      IBM_CUDA_TRY((launch_explicit<T, true>(g, u, v, w, pr, (T *)s->Nu, (T *)s->Nv, (T *)s->Nw, du, dv, dw, ab * nu,
+                                             ab, gm, zt, dt, v_lo, uo, vo, wo, st)));
     else
-      IBM_CUDA_TRY(launch_pdl(k_explicit<T, false>, eg, dim3(kExTX, kExTZ), 0, st, g, u, v, w, pr, (T *)s->Nu,
-                              (T *)s->Nv, (T *)s->Nw, du, dv, dw, (T)(ab * nu), (T)ab, (T)gm, (T)zt, (T)dt, (T)0,
-                              (const T *)nullptr, (const T *)nullptr, (const T *)nullptr));
+      IBM_CUDA_TRY((launch_explicit<T, false>(g, u, v, w, pr, (T *)s->Nu, (T *)s->Nv, (T *)s->Nw, du, dv, dw, ab * nu,
+                                              ab, gm, zt, dt, (T)0, nullptr, nullptr, nullptr, st)));
   }
   // L2 + L1
   if (nmk > 0) {

@@ -301,3 +301,30 @@ def test_substep_with_gather_spreading(prec):
     print("stage errors", errs)
     for k in ("u", "v", "w", "p"):
         assert np.array_equal(runs[0][k], runs[1][k]), k
+
+
+@pytest.mark.parametrize("shape", [(8, 9, 8), (12, 8, 24), (48, 13, 12), (64, 33, 8), (96, 17, 48)])
+@pytest.mark.parametrize("inout", [False, True])
+@pytest.mark.parametrize("prec", [ibm.IBM_FP64, ibm.IBM_FP32_REFINED])
+def test_explicit_terms_partial_tiles_and_chunks(shape, inout, prec):
+    """E1 marches 32 x 8 column tiles up chunks of y planes: tiles wider and
+    deeper than the grid, a last tile partly outside (its halo wraps inside the
+    tile), a last chunk of one plane, a chunk next to either wall."""
+    nx, ny, nz = shape
+    npdt = np.float64 if prec == ibm.IBM_FP64 else np.float32
+    dt_t = torch.float64 if prec == ibm.IBM_FP64 else torch.float32
+    tol = TOL_STAGE_FP64 if prec == ibm.IBM_FP64 else TOL_STAGE_FP32
+    g, (u, v, w, p), Np, X0, dV = _setup(nx, ny, nz, 40, npdt, wl=90 + nx)
+    params = (0.1, 0.0, 0.0)
+    st = dict(u=u, v=v, w=w, p=p, N_prev=tuple(Np), t=0.0)
+    mk = dict(X0=X0, dV=dV, kind=O.MOTION_TRANSLATE, params=params)
+    if inout:
+        io = _inout_data(nx, nz, npdt, 91)
+        ref, _ = O.rk_stage(st, mk, 2, 1e-3, 1e-2, g, inout=io)
+        got = _run_gpu_inout(g, [u, v, w, p], Np, X0, dV, io, [2], 1e-3, 1e-2, params, prec, dt_t)
+    else:
+        ref, _ = O.rk_stage(st, mk, 2, 1e-3, 1e-2, g)
+        got = _run_gpu(g, [u, v, w, p], Np, X0, dV, 2, 1e-3, 1e-2, ibm.IBM_MOTION_TRANSLATE, params, prec, dt_t, 0.0)
+    errs = {k: rel_err(got[k], ref[k]) for k in ("u", "v", "w", "p")}
+    errs.update({"N%d" % c: rel_err(got["N"][c], ref["N_prev"][c]) for c in range(3)})
+    assert stage_ok(errs, tol, tol if prec == ibm.IBM_FP64 else TOL_STAGE_FP32_N), errs
