@@ -69,7 +69,7 @@ k_rows_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__ 
   __syncthreads();
   for (int job = threadIdx.x; job < np * N1; job += NT) {
     const int p = job / N1, n1 = job - p * N1;
-    rfwd_step1<T, N>(in + (size_t)(pair0 + p) * 2 * N, n1, tw2, X + (p * N1 + n1) * PITCH);
+    rfwd_step1<T, N>(in + (size_t)(pair0 + p) * 2 * N, N, n1, tw2, X + (p * N1 + n1) * PITCH);
   }
   __syncthreads();
   if constexpr (!Cfg::LANE) {

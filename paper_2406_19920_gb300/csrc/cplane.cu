@@ -79,7 +79,7 @@ k_cplane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict_
     const int np = min(CP, R / 2 - p0);
     for (int job = tid; job < np * N1X; job += NT) {
       const int p = job / N1X, n1 = job - p * N1X;
-      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, n1, tw2x, X + (p * N1X + n1) * XPITCH);
+      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, NX, n1, tw2x, X + (p * N1X + n1) * XPITCH);
     }
     __syncthreads();
     for (int job = tid; job < np * J3; job += NT) {

@@ -191,13 +191,14 @@ __device__ __forceinline__ void load_step_twiddles(cplx<T> *tw2, const cplx<T> *
 // ---------------------------------------------------------------------------
 
 // Rows forward, step 1, lane n1 of one real row pair (a = rows[0, N),
-// b = rows[N, 2N)): z = a + i b; x = the lane's exchange row (N2 entries).
+// b = rows[pitch, pitch + N)): z = a + i b; x = the lane's exchange row (N2
+// entries).
 template <typename T, int N>
-__device__ __forceinline__ void rfwd_step1(const T *rows, int n1, const cplx<T> *tw2, cplx<T> *x) {
+__device__ __forceinline__ void rfwd_step1(const T *rows, int pitch, int n1, const cplx<T> *tw2, cplx<T> *x) {
   constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
   cplx<T> v[N2];
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) v[n2] = mk<T>(rows[n1 + N1 * n2], rows[N + n1 + N1 * n2]);
+  for (int n2 = 0; n2 < N2; ++n2) v[n2] = mk<T>(rows[n1 + N1 * n2], rows[pitch + n1 + N1 * n2]);
   reg_dft<false, N2>(v);
   x[0] = v[0];
 #pragma unroll

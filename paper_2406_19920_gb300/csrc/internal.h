@@ -235,6 +235,13 @@ bool slab_residual_fused(int nx, int nz);  // the pass exists for this x length 
 cudaError_t launch_slab_residual_forward(const StencilCoef &c, int nx, int ny, int nz, const float *b, const float *x,
                                          float2 *S, const float2 *twx, const double *boff, double *norms, int *err,
                                          cudaStream_t st);
+// The refinement's correction right-hand side r = b - A x and its forward
+// transform in one pass of the FP32 plane kernels (plane mode 1, every field
+// kind); r never reaches global memory.
+bool plane_residual_fused(const TransformGeom &g);
+cudaError_t launch_plane_residual_forward(const TransformGeom &g, const StencilCoef &c, const float *b, const float *x,
+                                          float2 *S, const float2 *twx, const float2 *twz, const double *boff,
+                                          cudaStream_t st);
 // dst plane jlo += clo g_lo, plane jhi += chi g_hi ([nz][nx] planes; NULL skips a side).
 template <typename T>
 cudaError_t launch_wall_rhs(int nx, int nz, T *dst, int jlo, int jhi, const T *glo, const T *ghi, double clo,

@@ -209,9 +209,12 @@ static bool slab_applies(const ibm_plan_s *p, const PencilParams &pp) {
   return p->use_slab && pp.j0 == 0 && pp.nb == 1 && !pp.periodic;
 }
 
+// res: the right-hand side is the refinement residual in - A res_x of these
+// coefficients, formed inside the forward transform (FP32 plane kernels).
 template <typename T>
 static int solve_once(ibm_plan_s *p, const PencilParams &pp, const T *in, T *out, const T *addend,
-                      double *mean_out, cudaStream_t st) {
+                      double *mean_out, cudaStream_t st, const StencilCoef *res = nullptr, const T *res_x = nullptr,
+                      const double *boff = nullptr) {
   if constexpr (sizeof(T) == 4) {
     if (slab_applies(p, pp)) return solve_once_slab(p, pp, in, out, addend, mean_out, st);
   }
@@ -225,7 +228,12 @@ static int solve_once(ibm_plan_s *p, const PencilParams &pp, const T *in, T *out
   const cplx<T> *twx = static_cast<const cplx<T> *>(p->twx);
   const cplx<T> *twz = static_cast<const cplx<T> *>(p->twz);
   const int nl = transform_launches<T>(g);
-  {
+  if (res) {
+    if constexpr (sizeof(T) == 4) {
+      ProfScope ps(p, IBM_K_RESIDUAL, st);
+      IBM_CUDA_TRY(launch_plane_residual_forward(gf, *res, in, res_x, S, twx, twz, boff, st));
+    }
+  } else {
     ProfScope ps(p, IBM_K_FORWARD, st, nl);
     IBM_CUDA_TRY(launch_forward<T>(gf, ptr3(in), ptr3(S), twx, twz, st));
   }
@@ -317,6 +325,11 @@ static int plan_solve_t(ibm_plan_s *p, int kind, double c, int field_bc, const T
                                                     kind == 0 ? p->dsc : nullptr, nullptr, p->derr, st));
         }
         rc = solve_once_slab(p, pp, nullptr, out, out, nullptr, st, 1);
+        if (rc) return rc;
+        continue;
+      }
+      if (!slab_applies(p, pp) && plane_residual_fused(geom_of(p))) {
+        rc = solve_once<T>(p, pp, b, out, out, nullptr, st, &sc, out, kind == 0 ? p->dsc : nullptr);
         if (rc) return rc;
         continue;
       }

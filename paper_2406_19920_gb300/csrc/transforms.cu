@@ -19,172 +19,39 @@
 //   axis kernels    (mode 0, axis.cu) x-rows and z-columns in two passes;
 //   cluster kernels (modes 2, 4, 8, cplane.cu) C CTAs per plane.
 // Plane and axis kernels run the two-step register transform of fft2.cuh.
-#include "fft2.cuh"
-#include "internal.h"
+#include "plane.cuh"
 
 namespace ibm {
-
-// --------------------------------------------------------------------------
-// plane kernels: one CTA per y-plane
-// --------------------------------------------------------------------------
-// Shared memory (complex entries): tw2x [NX], tw2z [NZ], the spectrum plane
-// [NZ][P], and one exchange buffer reused by the x chunks (CP row pairs,
-// [CP][N1x][N2x+1]) and the z chunks (CW columns, [N1z][N2z][CW]); chunk
-// sizes fill what the plane leaves of the 227 KB.
-template <typename T, int NX, int NZ> struct PlaneCfg {
-  using C = cplx<T>;
-  static constexpr int P = NX / 2 + 1;
-  static constexpr int N1X = TwoStep<NX>::N1, N2X = TwoStep<NX>::N2, XPITCH = N2X + 1;
-  static constexpr size_t fixed = sizeof(C) * ((size_t)NX + NZ + (size_t)NZ * P);
-  static constexpr size_t room = fixed < kPlaneSmemLimit ? kPlaneSmemLimit - fixed : 0;
-  static constexpr size_t pair_bytes = sizeof(C) * N1X * XPITCH;
-  static constexpr size_t col_bytes = sizeof(C) * NZ;
-  static constexpr int CP0 = (int)(room / pair_bytes), CW0 = (int)(room / col_bytes);
-  static constexpr int CP = CP0 < NZ / 2 ? CP0 : NZ / 2;
-  static constexpr int CW = CW0 < P ? CW0 : P;
-  static constexpr bool ok = CP >= (NZ / 2 < 8 ? NZ / 2 : 8) && CW >= (P < 8 ? P : 8);
-  static constexpr size_t xbytes = (size_t)CP * pair_bytes > (size_t)CW * col_bytes ? (size_t)CP * pair_bytes
-                                                                                    : (size_t)CW * col_bytes;
-  static constexpr size_t bytes = fixed + xbytes;
-  // threads: enough for the largest of the x step-1, x step-3 and z step-1
-  // job counts in one round (z step 3 takes N2z / N1z rounds), <= 1024
-  static constexpr int N1Z = TwoStep<NZ>::N1;
-  static constexpr int J3 = N2X / 2;
-  static constexpr int JMAX0 = CP * N1X > CP * J3 ? CP * N1X : CP * J3;
-  static constexpr int JMAX = JMAX0 > CW * N1Z ? JMAX0 : CW * N1Z;
-  static constexpr int THREADS = JMAX >= 1024 ? 1024 : (JMAX + 31) / 32 * 32;
-};
-
-template <typename T, int NX, int NZ>
-__global__ void __launch_bounds__(PlaneCfg<T, NX, NZ>::THREADS)
-k_plane_fwd(Ptr3<const T *> in_, Ptr3<cplx<T> *> S_, const cplx<T> *__restrict__ twx,
-            const cplx<T> *__restrict__ twz, double *zrhs) {
-  const T *__restrict__ in = in_[blockIdx.y];
-  cplx<T> *__restrict__ S = S_[blockIdx.y];
-  using Cfg = PlaneCfg<T, NX, NZ>;
-  constexpr int P = Cfg::P, N1X = Cfg::N1X, XPITCH = Cfg::XPITCH, CP = Cfg::CP, CW = Cfg::CW;
-  constexpr int kPlaneThreads_ = Cfg::THREADS;
-  constexpr int N1Z = TwoStep<NZ>::N1, N2Z = TwoStep<NZ>::N2, J3 = Cfg::N2X / 2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cplx<T> *tw2x = reinterpret_cast<cplx<T> *>(smem_raw);
-  cplx<T> *tw2z = tw2x + NX;
-  cplx<T> *plane = tw2z + NZ;  // [NZ][P]
-  cplx<T> *X = plane + NZ * P;
-  const int j = blockIdx.x;
-  const int tid = threadIdx.x;
-  load_step_twiddles<T, NX>(tw2x, twx);
-  load_step_twiddles<T, NZ>(tw2z, twz);
-  pdl_wait();  // the fields below are the predecessor's output
-  __syncthreads();
-  const T *src = in + (size_t)j * NZ * NX;
-  for (int p0 = 0; p0 < NZ / 2; p0 += CP) {
-    const int np = min(CP, NZ / 2 - p0);
-    for (int job = tid; job < np * N1X; job += kPlaneThreads_) {
-      const int p = job / N1X, n1 = job - p * N1X;
-      rfwd_step1<T, NX>(src + (size_t)(p0 + p) * 2 * NX, n1, tw2x, X + (p * N1X + n1) * XPITCH);
-    }
-    __syncthreads();
-    for (int job = tid; job < np * J3; job += kPlaneThreads_) {
-      const int p = job / J3, q = job - p * J3;
-      cplx<T> *dA = plane + (p0 + p) * 2 * P;
-      rfwd_step3<T, NX, XPITCH>(X + p * N1X * XPITCH, q, dA, dA + P);
-    }
-    __syncthreads();
-  }
-  cplx<T> *dst = S + (size_t)j * NZ * P;
-  for (int c0 = 0; c0 < P; c0 += CW) {
-    const int nc = min(CW, P - c0);
-    for (int job = tid; job < CW * N1Z; job += kPlaneThreads_) {
-      const int n1 = job / CW, c = job - n1 * CW;
-      if (c < nc)
-        col_step1<T, NZ, false, CW>(plane + c0 + c, P, n1, tw2z, X + n1 * N2Z * CW + c, false, mk<T>((T)0, (T)0));
-    }
-    __syncthreads();
-    for (int job = tid; job < CW * N2Z; job += kPlaneThreads_) {
-      const int k2 = job / CW, c = job - k2 * CW;
-      if (c < nc) {
-        const cplx<T> u0 = col_step3<T, NZ, false, CW>(X, c, k2, dst + c0 + c, P);
-        if (zrhs && c0 + c == 0 && k2 == 0) zrhs[j] = 0.5 * (double)u0.x;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Inverse: spectrum plane -> out = addend + scale * result.
-template <typename T, int NX, int NZ>
-__global__ void __launch_bounds__(PlaneCfg<T, NX, NZ>::THREADS)
-k_plane_inv(Ptr3<cplx<T> *> S_, Ptr3<T *> out_, Ptr3<const T *> add_, const cplx<T> *__restrict__ twx,
-            const cplx<T> *__restrict__ twz, T scale, const double *zsol) {
-  const cplx<T> *__restrict__ S = S_[blockIdx.y];
-  T *out = out_[blockIdx.y];
-  const T *addend = add_[blockIdx.y];
-  using Cfg = PlaneCfg<T, NX, NZ>;
-  constexpr int P = Cfg::P, N1X = Cfg::N1X, N2X = Cfg::N2X, XPITCH = Cfg::XPITCH, CP = Cfg::CP, CW = Cfg::CW;
-  constexpr int kPlaneThreads_ = Cfg::THREADS;
-  constexpr int N1Z = TwoStep<NZ>::N1, N2Z = TwoStep<NZ>::N2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cplx<T> *tw2x = reinterpret_cast<cplx<T> *>(smem_raw);
-  cplx<T> *tw2z = tw2x + NX;
-  cplx<T> *plane = tw2z + NZ;
-  cplx<T> *X = plane + NZ * P;
-  const int j = blockIdx.x;
-  const int tid = threadIdx.x;
-  load_step_twiddles<T, NX>(tw2x, twx);
-  load_step_twiddles<T, NZ>(tw2z, twz);
-  pdl_wait();  // the fields below are the predecessor's output
-  __syncthreads();
-  const cplx<T> *src = S + (size_t)j * NZ * P;
-  const cplx<T> z0 = zsol ? mk<T>((T)(2.0 * zsol[j]), (T)0) : mk<T>((T)0, (T)0);
-  for (int c0 = 0; c0 < P; c0 += CW) {
-    const int nc = min(CW, P - c0);
-    for (int job = tid; job < CW * N1Z; job += kPlaneThreads_) {
-      const int n1 = job / CW, c = job - n1 * CW;
-      if (c < nc)
-        col_step1<T, NZ, true, CW>(src + c0 + c, P, n1, tw2z, X + n1 * N2Z * CW + c, zsol && c0 + c == 0, z0);
-    }
-    __syncthreads();
-    for (int job = tid; job < CW * N2Z; job += kPlaneThreads_) {
-      const int k2 = job / CW, c = job - k2 * CW;
-      if (c < nc) col_step3<T, NZ, true, CW>(X, c, k2, plane + c0 + c, P);
-    }
-    __syncthreads();
-  }
-  T *dst = out + (size_t)j * NZ * NX;
-  const T *add = addend ? addend + (size_t)j * NZ * NX : nullptr;
-  for (int p0 = 0; p0 < NZ / 2; p0 += CP) {
-    const int np = min(CP, NZ / 2 - p0);
-    for (int job = tid; job < np * N1X; job += kPlaneThreads_) {
-      const int p = job / N1X, n1 = job - p * N1X;
-      const cplx<T> *sA = plane + (p0 + p) * 2 * P;
-      rinv_step1<T, NX>(sA, sA + P, n1, tw2x, X + (p * N1X + n1) * XPITCH);
-    }
-    __syncthreads();
-    for (int job = tid; job < np * N2X; job += kPlaneThreads_) {
-      const int p = job / N2X, k2 = job - p * N2X;
-      const size_t r = (size_t)(p0 + p) * 2 * NX;
-      rinv_step3<T, NX, XPITCH>(X + p * N1X * XPITCH, k2, dst + r, dst + r + NX, add ? add + r : nullptr,
-                                add ? add + r + NX : nullptr, scale);
-    }
-    __syncthreads();
-  }
-}
 
 // --------------------------------------------------------------------------
 // dispatch
 // --------------------------------------------------------------------------
 #define IBM_FOR_EACH_N(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512)
 
-// plane kernels are instantiated for square-ish planes whose spectrum fits in shared memory
+// FP64 plane kernels (the tuner's; FP32: plane.cuh)
 #define IBM_PLANE_SHAPES(X)                                                    \
   X(8, 8) X(12, 12) X(16, 16) X(24, 24) X(32, 32) X(48, 48) X(64, 64) X(96, 96) \
   X(128, 128) X(192, 192) X(256, 128) X(128, 256) X(64, 128) X(128, 64)
 
 template <typename T> static bool plane_supported(int nx, int nz) {
-#define X(a, b) if (nx == a && nz == b) return PlaneCfg<T, a, b>::ok;
-  IBM_PLANE_SHAPES(X)
+  if constexpr (sizeof(T) == 4) {
+#define X(N) if (nx == N) return plane_dispatch<N>(nz, [](auto) {}, PlaneLengths{});
+    IBM_FOR_EACH_N(X)
 #undef X
+  } else {
+#define X(a, b) if (nx == a && nz == b) return PlaneCfg<T, a, b>::ok;
+    IBM_PLANE_SHAPES(X)
+#undef X
+  }
   return false;
+}
+
+static cudaError_t plane_forward(const TransformGeom &g, Ptr3<const float *> in, Ptr3<float2 *> S, const float2 *twx,
+                                 const float2 *twz, const PlaneResidual &res, cudaStream_t st) {
+#define X(N) if (g.nx == N) return plane_forward_f32<N>(g, in, S, twx, twz, res, st);
+  IBM_FOR_EACH_N(X)
+#undef X
+  return cudaErrorNotSupported;
 }
 
 template <typename T>
@@ -197,19 +64,32 @@ cudaError_t launch_forward(const TransformGeom &g, Ptr3<const T *> in, Ptr3<cplx
   if (g.use_plane >= 2 && cplane_supported<T>(nx, nz, g.use_plane))
     return launch_cplane_forward<T>(g, g.use_plane, in, S, twx, twz, st);
   if (g.use_plane == 1 && plane_supported<T>(nx, nz)) {
+    if constexpr (sizeof(T) == 4) {
+      return plane_forward(g, in, S, twx, twz, PlaneResidual{}, st);
+    } else {
 #define X(a, b)                                                                                  \
   if (nx == a && nz == b) {                                                                      \
     if constexpr (PlaneCfg<T, a, b>::ok) {                                                       \
       { cudaError_t e = ensure_max_smem<k_plane_fwd<T, a, b>>(); if (e) return e; }              \
-      IBM_KTRY(launch_pdl(k_plane_fwd<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, in, S, twx, twz, g.zrhs)); \
+      IBM_KTRY(launch_pdl(k_plane_fwd<T, a, b>, dim3(ny, g.nb), PlaneCfg<T, a, b>::THREADS, PlaneCfg<T, a, b>::bytes, st, in, S, twx, twz, g.zrhs, PlaneResidual{})); \
       return cudaGetLastError();                                                                 \
     }                                                                                            \
   }
-    IBM_PLANE_SHAPES(X)
+      IBM_PLANE_SHAPES(X)
 #undef X
+    }
   }
   // axis path: x rows then z columns
   return launch_axis_forward<T>(g, in, S, twx, twz, st);
+}
+
+bool plane_residual_fused(const TransformGeom &g) { return g.use_plane == 1 && plane_supported<float>(g.nx, g.nz); }
+
+cudaError_t launch_plane_residual_forward(const TransformGeom &g, const StencilCoef &c, const float *b, const float *x,
+                                          float2 *S, const float2 *twx, const float2 *twz, const double *boff,
+                                          cudaStream_t st) {
+  const PlaneResidual res{x, make_args(g.nx, g.ny, g.nz, c, boff)};
+  return plane_forward(g, ptr3(b), ptr3(S), twx, twz, res, st);
 }
 
 template <typename T>
@@ -222,6 +102,11 @@ cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> 
   if (g.use_plane >= 2 && cplane_supported<T>(nx, nz, g.use_plane))
     return launch_cplane_inverse<T>(g, g.use_plane, S, out, addend, twx, twz, scale, st);
   if (g.use_plane == 1 && plane_supported<T>(nx, nz)) {
+    if constexpr (sizeof(T) == 4) {
+#define X(N) if (nx == N) return plane_inverse_f32<N>(g, S, out, addend, twx, twz, scale, st);
+      IBM_FOR_EACH_N(X)
+#undef X
+    } else {
 #define X(a, b)                                                                                  \
   if (nx == a && nz == b) {                                                                      \
     if constexpr (PlaneCfg<T, a, b>::ok) {                                                       \
@@ -230,8 +115,9 @@ cudaError_t launch_inverse(const TransformGeom &g, Ptr3<cplx<T> *> S, Ptr3<T *> 
       return cudaGetLastError();                                                                 \
     }                                                                                            \
   }
-    IBM_PLANE_SHAPES(X)
+      IBM_PLANE_SHAPES(X)
 #undef X
+    }
   }
   return launch_axis_inverse<T>(g, S, out, addend, twx, twz, scale, st);
 }
@@ -267,13 +153,26 @@ template int plane_modes<float>(int, int, int *);
 template int plane_modes<double>(int, int, int *);
 
 template <typename T> int default_plane_mode(int nx, int ny, int nz) {
-  // Measured on GB300 (128^3 to 384x256x256): in FP32 the one-CTA plane
-  // kernels win up to 128 x 256 planes and the split passes from 192^2 on;
-  // in FP64 (arithmetic-bound here) the split passes win at every size.
-  // The cluster kernels lose to both and stay available to the tuner and to
-  // IBM_PLANE_MODE.
-  (void)ny;
-  if (sizeof(T) == 4 && plane_supported<T>(nx, nz) && nx * nz <= 128 * 256) return 1;
+  // FP64 (arithmetic-bound) takes the split passes at every size, and so does
+  // FP32 beyond the planes below.  Measured on GB300 over 40 plane shapes and ny
+  // = 8 .. 512 (refined FP32 solve, split passes against plane kernels with the
+  // residual in the forward transform, us):
+  //   small planes win by their launches (6 against 11) and at any ny where the
+  //   rows are short: 48x33x24 28.5 / 17, 64x512x64 60 / 53, 128x512x64 80 / 75;
+  //   with long rows up to one CTA an SM: 256x129x32 39 / 32, 256x512x32 77 / 92;
+  //   middle planes from about a third of the SMs on: 96x33x96 30.9 / 31.8,
+  //   96x64x96 33.1 / 31.2, 96x512x96 96 / 87;
+  //   large planes (one CTA an SM) where their CTAs fill one wave of the SMs, or
+  //   two with short rows: 128x64x128 37.7 / 39.2, 128x129x128 54 / 44,
+  //   192x129x96 58 / 47, 192x256x128 128 / 117, 128x512x128 159 / 168,
+  //   256x16x128 33 / 61.
+  if (sizeof(T) == 4 && plane_supported<T>(nx, nz)) {
+    const int area = nx * nz;
+    const bool wave = (ny >= 80 && ny <= 152) || (nx <= 192 && ny >= 240 && ny <= 304);
+    if (area <= 8192) return ny <= 152 || (nx <= 192 && nz <= 256);
+    if (area <= 12288) return wave || (nx <= 192 && nz <= 192 && ny >= 56);
+    if (area <= kPlaneArea) return wave;
+  }
   return 0;
 }
 template int default_plane_mode<float>(int, int, int);
