@@ -475,10 +475,16 @@ k_pencil_seg(Ptr3<cplx<T> *> S_, const T *__restrict__ lamx, const T *__restrict
   T *ws = reinterpret_cast<T *>(tile + (size_t)(L * S + 1) * 32);  // [L S][32] w of every row
   T *cf = ws + (size_t)L * S * 32;  // [4][L][32] (yhat_end.x, .y, prod w, q of the last row)
   T *cb = cf + 4 * L * 32;          // [2][L][32] (xhat_first.x, .y)
-  const int G = gridDim.x - (pp.zero_mode ? 1 : 0);
-  if (pp.zero_mode && blockIdx.x == G) {
+  // CTA 0 takes the zero mode: a long FP64 chain, so it starts with the
+  // others, on a place of its own (as the last CTA of a full grid it waited
+  // for a resident one to end: Poisson 384 x 200 x 192 34.7 -> 33.8 us)
+  const int zc = pp.zero_mode ? 1 : 0;
+  const int G = gridDim.x - zc;
+  if (zc && blockIdx.x == 0) {
     pdl_wait();
-    zero_mode_cta(pp, reinterpret_cast<double *>(cb + 2 * L * 32), mean_out);
+    if (threadIdx.x < 32)
+      zero_mode_fp64(pp.zrhs, pp.zsol, reinterpret_cast<double *>(cb + 2 * L * 32), pp.ny, pp.inv_ny, pp.hy2,
+                     pp.inv_nxnz, mean_out);
     return;
   }
   const long plane = (long)pp.nz * pp.P;
@@ -491,7 +497,7 @@ k_pencil_seg(Ptr3<cplx<T> *> S_, const T *__restrict__ lamx, const T *__restrict
   cplx<T> *tm = tile + (size_t)L * S * 32 + lane;
   T *wc = ws + (size_t)seg * S * 32 + lane;  // w of my row u at wc[32 u]
   pdl_wait();
-  int t = blockIdx.x;
+  int t = blockIdx.x - zc;
   if (t < tiles) seg_issue<T, S>(seg_tile<T, S>(pp, S_, lamx, lamz, t, nblk, seg, lane, Lh), tl, tm, seg, plane);
   for (; t < tiles; t += G) {
     const SegTile<T> cur = seg_tile<T, S>(pp, S_, lamx, lamz, t, nblk, seg, lane, Lh);
@@ -595,19 +601,26 @@ static cudaError_t launch_seg(const PencilParams &pp, Ptr3<cplx<T> *> S3, const 
   int per_sm = 0;
   IBM_KTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pencil_seg<T, S, MAXT>, 32 * L, bytes));
   const int tiles = ceil_div(pp.nz * pp.P, 32) * pp.nb;
-  const int G = std::max(1, std::min(tiles, sms * std::max(per_sm, 1)));
-  IBM_KTRY(launch_pdl(k_pencil_seg<T, S, MAXT>, G + (pp.zero_mode ? 1 : 0), 32 * L, bytes, st, S3, lamx, lamz, pp,
+  const int zc = pp.zero_mode ? 1 : 0;
+  const int G = std::max(1, std::min(tiles, sms * std::max(per_sm, 1) - zc));
+  IBM_KTRY(launch_pdl(k_pencil_seg<T, S, MAXT>, G + zc, 32 * L, bytes, st, S3, lamx, lamz, pp,
                       mean_out));
   return cudaGetLastError();
 }
 
 // Rows per warp of the segmented sweep for ny rows (0: not available; the
 // CTA has 2 ceil((ny / 2) / S) warps).
-template <typename T> static int seg_rows(int ny) {
+// fast: every pencil's pivots converge within a 16-row segment (see
+// launch_pencil).  FP32, 129 to 256 rows: 16-row segments on up to 16 warps, one
+// CTA an SM, where all segments but the first run with constant pivots (three
+// fields of a stage at 384 x 256 x 256 140 -> 128 us, Helmholtz 192 x 129 x 96 11.3
+// -> 7.6 us), else 32-row segments on 8 warps, two CTAs (Poisson 384 x 256 x 192
+// 36 against 38 us).
+template <typename T> static int seg_rows(int ny, bool fast) {
   if (ny < 4) return 0;
   if (ny <= 64) return 8;
   if (ny <= 128) return 16;
-  if (ny <= 256) return sizeof(T) == 4 ? 32 : 16;
+  if (ny <= 256) return sizeof(T) == 4 && !fast ? 32 : 16;
   return (sizeof(T) == 4 && ny <= 512) ? 32 : 0;
 }
 
@@ -998,10 +1011,15 @@ cudaError_t launch_pencil(const PencilParams &pp, Ptr3<cplx<T> *> S3, const T *l
   }
   // default: the segmented sweep for FP32 (measured faster at 128^3 and
   // 256^3); FP64 is bound by its divisions and stays on the two-ended sweep
-  if (pp.mode == 4 || (pp.mode == 0 && sizeof(T) == 4 && seg_rows<T>(pp.ny) > 0)) {
-    switch (seg_rows<T>(pp.ny)) {
+  if (pp.mode == 4 || (pp.mode == 0 && sizeof(T) == 4 && seg_rows<T>(pp.ny, false) > 0)) {
+    // e_k - e+ shrinks by w^2 a row, w + 1 / w = 2 + g / a: with g / a >= 0.4, w^2 <= 0.29 and 16 rows take
+    // it below 2^-28
+    const bool fast = pp.g_add >= 0.4 * pp.a;
+    switch (seg_rows<T>(pp.ny, fast)) {
       case 8: return launch_seg<T, 8, 256>(pp, S3, lamx, lamz, mean_out, st);
-      case 16: return launch_seg<T, 16, sizeof(T) == 4 ? 256 : 512>(pp, S3, lamx, lamz, mean_out, st);
+      case 16:
+        if (sizeof(T) == 4 && pp.ny <= 128) return launch_seg<T, 16, 256>(pp, S3, lamx, lamz, mean_out, st);
+        return launch_seg<T, 16, 512>(pp, S3, lamx, lamz, mean_out, st);
       case 32:
         if constexpr (sizeof(T) == 4) {
           if (pp.ny <= 256) return launch_seg<T, 32, 256>(pp, S3, lamx, lamz, mean_out, st);

@@ -413,3 +413,26 @@ def test_fp64_sweeps_constant_from_the_converged_row(ny, mode, monkeypatch):
                 assert rel_err(host(x), O.helmholtz_solve(bb, g, c, bc)) <= tol, (c, bc)
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("ny", [129, 144, 145, 255, 256])
+@pytest.mark.parametrize("c", [2e-6, 1e-4, 5.0])
+def test_fp32_segments_of_129_to_256_rows(ny, c):
+    """FP32 pencils of 129 to 256 rows take 16-row segments where their pivots
+    converge within one (small c) and 32-row segments otherwise; whole and
+    partial last segments, the three wall kinds, beside the Poisson solve."""
+    g = grid(32, ny, 24)
+    b = synth.white_noise(32, ny, 24, workload=17, stream=ny).astype(np.float32).astype(np.float64)
+    plan = _plan(32, ny, 24, g, ibm.IBM_FP32_REFINED)
+    try:
+        x = torch.empty(b.shape, dtype=torch.float32, device="cuda")
+        ibm.ibm_poisson_solve(plan, dev(b, torch.float32), x)
+        assert rel_err(host(x), O.poisson_solve(b, g)[0]) <= TOL_FP32
+        for bc in (O.NEUMANN, O.CELL_DIRICHLET, O.FACE_DIRICHLET):
+            bb = b.copy()
+            if bc == O.FACE_DIRICHLET:
+                bb[0] = 0.0
+            ibm.ibm_helmholtz_solve(plan, c, bc, dev(bb, torch.float32), x)
+            assert rel_err(host(x), O.helmholtz_solve(bb, g, c, bc)) <= TOL_FP32, bc
+    finally:
+        ibm.ibm_plan_destroy(plan)
