@@ -77,20 +77,20 @@ template <bool INV, typename C> __device__ __forceinline__ void dft8(C *v) {
   C o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
   dft4<INV>(e0, e1, e2, e3);
   dft4<INV>(o0, o1, o2, o3);
-  // o_k *= W8^k (fwd: exp(-i pi k / 4))
-  C w1, w3;
+  // o_k *= W8^k (fwd: exp(-i pi k / 4)); the factor s goes into the last additions
+  C w1, w3;  // W8 o1 / s, W8^3 o3 / s
   if (INV) {
-    w1.x = s * (o1.x - o1.y); w1.y = s * (o1.x + o1.y);      // (1+i)/sqrt2
-    w3.x = -s * (o3.x + o3.y); w3.y = s * (o3.x - o3.y);     // (-1+i)/sqrt2
+    w1.x = o1.x - o1.y; w1.y = o1.x + o1.y;      // (1+i)
+    w3.x = -(o3.x + o3.y); w3.y = o3.x - o3.y;   // (-1+i)
   } else {
-    w1.x = s * (o1.x + o1.y); w1.y = s * (o1.y - o1.x);      // (1-i)/sqrt2
-    w3.x = s * (o3.y - o3.x); w3.y = -s * (o3.x + o3.y);     // (-1-i)/sqrt2
+    w1.x = o1.x + o1.y; w1.y = o1.y - o1.x;      // (1-i)
+    w3.x = o3.y - o3.x; w3.y = -(o3.x + o3.y);   // (-1-i)
   }
   C w2 = cmul_mi<INV>(o2);
   v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-  v[1] = cadd(e1, w1); v[5] = csub(e1, w1);
+  v[1].x = fma(s, w1.x, e1.x); v[1].y = fma(s, w1.y, e1.y); v[5].x = fma(-s, w1.x, e1.x); v[5].y = fma(-s, w1.y, e1.y);
   v[2] = cadd(e2, w2); v[6] = csub(e2, w2);
-  v[3] = cadd(e3, w3); v[7] = csub(e3, w3);
+  v[3].x = fma(s, w3.x, e3.x); v[3].y = fma(s, w3.y, e3.y); v[7].x = fma(-s, w3.x, e3.x); v[7].y = fma(-s, w3.y, e3.y);
 }
 
 template <int R, bool INV, typename C> __device__ __forceinline__ void dft(C *v) {

@@ -94,6 +94,66 @@ template <bool INV, int M, int N, typename C> __device__ __forceinline__ C twidd
   }
 }
 
+// x W_N^M up to a real factor in (0.7, 1]: the product is FACTOR * value.  With
+// the larger of cos and sin taken out, a rotation is two FMAs (t the ratio, at
+// most 1), and the factor goes into the additions that follow.
+template <bool INV, int M, int N> struct Rotation {
+  static constexpr int m = ((M % N) + N) % N;
+  static constexpr ctrig::CS w = ctrig::cs_turn(m, N);
+  static constexpr double s = INV ? -w.s : w.s;  // the factor of x is c - i s
+  static constexpr bool by_cos = w.c * w.c >= w.s * w.s;
+  static constexpr double factor = by_cos ? w.c : s;
+  static constexpr double t = by_cos ? s / w.c : w.c / s;
+  template <typename C> static __device__ __forceinline__ C apply(C x) {
+    using T = decltype(x.x);
+    constexpr T r = (T)t;
+    if (by_cos) return mk<T>(fma(r, x.y, x.x), fma(-r, x.x, x.y));  // (x c + y s, y c - x s) / c
+    return mk<T>(fma(r, x.x, x.y), fma(r, x.y, -x.x));              // the same / s
+  }
+};
+// (the exact angles: 0, a quarter, a half, three quarters of a turn)
+template <bool INV, int M, int N> constexpr bool exact_angle() { return (4 * ((M % N + N) % N)) % N == 0; }
+
+// The DFT of (u0, W^k u1, W^2k u2, W^3k u3), W = W_N, with the factors of the
+// rotations folded into the butterflies: 22 FMAs where rotating first takes 28
+// operations.
+template <bool INV, int K, int N, typename C> __device__ __forceinline__ void dft4_rotated(C &u0, C &u1, C &u2, C &u3) {
+  using T = decltype(u0.x);
+  if constexpr (exact_angle<INV, K, N>()) {
+    u1 = twiddle_const<INV, K, N>(u1);
+    u2 = twiddle_const<INV, 2 * K, N>(u2);
+    u3 = twiddle_const<INV, 3 * K, N>(u3);
+    dft4<INV>(u0, u1, u2, u3);
+  } else {
+    using R1 = Rotation<INV, K, N>;
+    using R3 = Rotation<INV, 3 * K, N>;
+    C t0, t1;
+    if constexpr (exact_angle<INV, 2 * K, N>()) {
+      const C r2 = twiddle_const<INV, 2 * K, N>(u2);
+      t0 = cadd(u0, r2);
+      t1 = csub(u0, r2);
+    } else {
+      using R2 = Rotation<INV, 2 * K, N>;
+      constexpr T f2 = (T)R2::factor;
+      const C r2 = R2::apply(u2);
+      t0 = mk<T>(fma(f2, r2.x, u0.x), fma(f2, r2.y, u0.y));
+      t1 = mk<T>(fma(-f2, r2.x, u0.x), fma(-f2, r2.y, u0.y));
+    }
+    constexpr bool x3 = exact_angle<INV, 3 * K, N>();
+    constexpr T f1 = (T)R1::factor, q = (T)((x3 ? 1.0 : R3::factor) / R1::factor);
+    const C r1 = R1::apply(u1);
+    C r3;
+    if constexpr (x3) r3 = twiddle_const<INV, 3 * K, N>(u3);
+    else r3 = R3::apply(u3);
+    const C a = mk<T>(fma(q, r3.x, r1.x), fma(q, r3.y, r1.y));
+    const C b = cmul_mi<INV>(mk<T>(fma(-q, r3.x, r1.x), fma(-q, r3.y, r1.y)));
+    u0 = mk<T>(fma(f1, a.x, t0.x), fma(f1, a.y, t0.y));
+    u2 = mk<T>(fma(-f1, a.x, t0.x), fma(-f1, a.y, t0.y));
+    u1 = mk<T>(fma(f1, b.x, t1.x), fma(f1, b.y, t1.y));
+    u3 = mk<T>(fma(-f1, b.x, t1.x), fma(-f1, b.y, t1.y));
+  }
+}
+
 template <bool INV, int N, typename C> __device__ __forceinline__ void reg_dft(C *v);
 
 // v[0..R*M) in natural order -> DFT in natural order (R M = N)
@@ -108,18 +168,19 @@ template <bool INV, int R, int M, typename C> __device__ __forceinline__ void re
     reg_dft<INV, M>(t);
     static_for<0, M>([&](auto i2) {
       constexpr int k2 = decltype(i2)::value;
-      y[n1 * M + k2] = twiddle_const<INV, n1 * k2, N>(t[k2]);
+      y[n1 * M + k2] = R == 4 ? t[k2] : twiddle_const<INV, n1 * k2, N>(t[k2]);
     });
   });
-#pragma unroll
-  for (int k2 = 0; k2 < M; ++k2) {
+  static_for<0, M>([&](auto i2) {
+    constexpr int k2 = decltype(i2)::value;
     C u[R];
 #pragma unroll
     for (int n1 = 0; n1 < R; ++n1) u[n1] = y[n1 * M + k2];
-    reg_dft<INV, R>(u);
+    if constexpr (R == 4) dft4_rotated<INV, k2, N>(u[0], u[1], u[2], u[3]);
+    else reg_dft<INV, R>(u);
 #pragma unroll
     for (int k1 = 0; k1 < R; ++k1) v[k2 + M * k1] = u[k1];
-  }
+  });
 }
 
 template <bool INV, int N, typename C> __device__ __forceinline__ void reg_dft(C *v) {
