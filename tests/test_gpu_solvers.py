@@ -436,3 +436,24 @@ def test_fp32_segments_of_129_to_256_rows(ny, c):
             assert rel_err(host(x), O.helmholtz_solve(bb, g, c, bc)) <= TOL_FP32, bc
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("ny", [8, 31, 65, 257])
+@pytest.mark.parametrize("bc", [O.NEUMANN, O.CELL_DIRICHLET, O.FACE_DIRICHLET])
+def test_residual_pass_marches_every_plane(ny, bc, monkeypatch):
+    """The FP32 residual pass of the split passes marches chunks of y planes:
+    refined solves with one chunk a plane up to long chunks and a short last
+    one, every wall kind."""
+    monkeypatch.setenv("IBM_PLANE_MODE", "0")
+    g = grid(128, ny, 96)
+    b = synth.white_noise(128, ny, 96, workload=18, stream=ny).astype(np.float32).astype(np.float64)
+    if bc == O.FACE_DIRICHLET:
+        b[0] = 0.0
+    plan = _plan(128, ny, 96, g, ibm.IBM_FP32_REFINED)
+    try:
+        x = torch.empty(b.shape, dtype=torch.float32, device="cuda")
+        info = ibm.ibm_helmholtz_solve(plan, 0.01, bc, dev(b, torch.float32), x, info=True)
+        assert rel_err(host(x), O.helmholtz_solve(b, g, 0.01, bc)) <= TOL_FP32
+        assert info["rel_residual"] < 1e-3
+    finally:
+        ibm.ibm_plan_destroy(plan)
