@@ -242,9 +242,10 @@ bool plane_residual_fused(const TransformGeom &g);
 cudaError_t launch_plane_residual_forward(const TransformGeom &g, const StencilCoef &c, const float *b, const float *x,
                                           float2 *S, const float2 *twx, const float2 *twz, const double *boff,
                                           cudaStream_t st);
-// dst plane jlo += clo g_lo, plane jhi += chi g_hi ([nz][nx] planes; NULL skips a side).
+// dst = src with clo g_lo added to plane jlo and chi g_hi to plane jhi ([nz][nx]
+// planes; NULL skips a side); everything 16-byte aligned.
 template <typename T>
-cudaError_t launch_wall_rhs(int nx, int nz, T *dst, int jlo, int jhi, const T *glo, const T *ghi, double clo,
-                            double chi, cudaStream_t st);
+cudaError_t launch_wall_rhs(int nx, int ny, int nz, const T *src, T *dst, int jlo, int jhi, const T *glo, const T *ghi,
+                            double clo, double chi, cudaStream_t st);
 
 }  // namespace ibm

@@ -449,13 +449,14 @@ static int solve_bc(ibm_plan_s *p, int kind, double c, int field_bc, const void 
   if (fb == IBM_FIELD_CELL_NEUMANN) { blo = -1.0 / hy; bhi = 1.0 / hy; }
   else if (fb == IBM_FIELD_CELL_DIRICHLET) { blo = bhi = 2.0 / (hy * hy); }
   else { blo = bhi = 1.0 / (hy * hy); jlo = 1; }
-  IBM_CUDA_TRY(cudaMemcpyAsync(p->bsave, rhs, p->npts * p->esz, cudaMemcpyDeviceToDevice, st));
   if (p->precision == IBM_FP64)
-    IBM_CUDA_TRY(launch_wall_rhs<double>(p->nx, p->nz, static_cast<double *>(p->bsave), jlo, jhi,
+    IBM_CUDA_TRY(launch_wall_rhs<double>(p->nx, p->ny, p->nz, static_cast<const double *>(rhs),
+                                         static_cast<double *>(p->bsave), jlo, jhi,
                                          static_cast<const double *>(glo), static_cast<const double *>(ghi),
                                          -tau * blo, -tau * bhi, st));
   else
-    IBM_CUDA_TRY(launch_wall_rhs<float>(p->nx, p->nz, static_cast<float *>(p->bsave), jlo, jhi,
+    IBM_CUDA_TRY(launch_wall_rhs<float>(p->nx, p->ny, p->nz, static_cast<const float *>(rhs),
+                                        static_cast<float *>(p->bsave), jlo, jhi,
                                         static_cast<const float *>(glo), static_cast<const float *>(ghi),
                                         -tau * blo, -tau * bhi, st));
   const int rc = plan_solve(p, kind, c, field_bc, p->bsave, out, nullptr, st, info);

@@ -169,31 +169,47 @@ cudaError_t launch_residual<float>(int nx, int ny, int nz, const StencilCoef &c,
 
 // Wall data's share of the 7-point operator, moved to the right-hand side
 // (Appendix B: the first and last rows of each pencil carry the boundary
-// values; BC2.2 forms the same terms from the FFT of the ghost planes).
-// dst[jlo] += clo g_lo, dst[jhi] += chi g_hi over one x-z plane each (either
-// g may be NULL).  One thread per plane point.
+// values; BC2.2 forms the same terms from the FFT of the ghost planes): dst =
+// src, with clo g_lo added to plane jlo and chi g_hi to plane jhi (either g may
+// be NULL).  16 bytes per thread; nx % 4 == 0, so no thread straddles planes.
+// (A copy and a launch over the two planes took 7 us at 192 x 129 x 96: solve 56.5 -> 52.2 us.)
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_wall_rhs(int npl, T *dst, size_t plane, int jlo, int jhi, const T *glo, const T *ghi, T clo, T chi) {
+k_wall_rhs(size_t nvec, const T *__restrict__ src, T *__restrict__ dst, int vplane, int jlo, int jhi,
+           const T *__restrict__ glo, const T *__restrict__ ghi, T clo, T chi) {
+  constexpr int V = 16 / sizeof(T);
+  struct alignas(16) Vec { T v[V]; };
   pdl_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= npl) return;
-  if (glo) dst[(size_t)jlo * plane + i] += clo * glo[i];
-  if (ghi) dst[(size_t)jhi * plane + i] += chi * ghi[i];
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nvec) return;
+  Vec x = reinterpret_cast<const Vec *>(src)[e];
+  auto add = [&](const T *g, int j, T c) {
+    const size_t e0 = (size_t)j * vplane;
+    if (g && e >= e0 && e < e0 + vplane) {
+      const Vec w = reinterpret_cast<const Vec *>(g)[e - e0];
+#pragma unroll
+      for (int q = 0; q < V; ++q) x.v[q] += c * w.v[q];
+    }
+  };
+  add(glo, jlo, clo);
+  add(ghi, jhi, chi);
+  reinterpret_cast<Vec *>(dst)[e] = x;
 }
 
 template <typename T>
-cudaError_t launch_wall_rhs(int nx, int nz, T *dst, int jlo, int jhi, const T *glo, const T *ghi, double clo,
-                            double chi, cudaStream_t st) {
-  const int npl = nx * nz;
-  IBM_KTRY(launch_pdl(k_wall_rhs<T>, ceil_div(npl, 256), 256, 0, st, npl, dst, (size_t)npl, jlo, jhi, glo, ghi,
-                      (T)clo, (T)chi));
+cudaError_t launch_wall_rhs(int nx, int ny, int nz, const T *src, T *dst, int jlo, int jhi, const T *glo, const T *ghi,
+                            double clo, double chi, cudaStream_t st) {
+  constexpr int V = 16 / sizeof(T);
+  const int vplane = nx * nz / V;
+  const size_t nvec = (size_t)vplane * ny;
+  IBM_KTRY(launch_pdl(k_wall_rhs<T>, (unsigned)((nvec + 255) / 256), 256, 0, st, nvec, src, dst, vplane, jlo, jhi, glo,
+                      ghi, (T)clo, (T)chi));
   return cudaGetLastError();
 }
-template cudaError_t launch_wall_rhs<float>(int, int, float *, int, int, const float *, const float *, double, double,
-                                            cudaStream_t);
-template cudaError_t launch_wall_rhs<double>(int, int, double *, int, int, const double *, const double *, double,
-                                             double, cudaStream_t);
+template cudaError_t launch_wall_rhs<float>(int, int, int, const float *, float *, int, int, const float *,
+                                            const float *, double, double, cudaStream_t);
+template cudaError_t launch_wall_rhs<double>(int, int, int, const double *, double *, int, int, const double *,
+                                             const double *, double, double, cudaStream_t);
 
 template <>
 cudaError_t launch_residual<double>(int nx, int ny, int nz, const StencilCoef &c, const double *b, const double *x,
