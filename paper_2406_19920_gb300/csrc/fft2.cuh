@@ -333,14 +333,12 @@ __device__ __forceinline__ void rfwd_step3_lane(const cplx<T> *xp, int t, bool l
   if (t == 0) split_put(u[N1 / 2], u[N1 / 2], dA + N / 2, dB + N / 2);
 }
 
-// Rows inverse, step 1, lane n1: Z_n = A_n + i B_n from the half spectra
-// sA, sB (n <= N/2; imaginary parts of bins 0 and N/2 dropped) and their
-// Hermitian extension for n > N/2.
+// Rows inverse, lane n1: its step-1 inputs Z_n = A_n + i B_n, n = n1 + N1 n2,
+// from the half spectra sA, sB (n <= N/2; imaginary parts of bins 0 and N/2
+// dropped) and their Hermitian extension for n > N/2.
 template <typename T, int N>
-__device__ __forceinline__ void rinv_step1(const cplx<T> *sA, const cplx<T> *sB, int n1, const cplx<T> *tw2,
-                                           cplx<T> *x) {
+__device__ __forceinline__ void rinv_load(const cplx<T> *sA, const cplx<T> *sB, int n1, cplx<T> (&v)[TwoStep<N>::N2]) {
   constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
-  cplx<T> v[N2];
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) {
     const int n = n1 + N1 * n2;
@@ -353,6 +351,14 @@ __device__ __forceinline__ void rinv_step1(const cplx<T> *sA, const cplx<T> *sB,
       v[n2] = mk<T>(a.x + b.y, b.x - a.y);
     }
   }
+}
+// Step 1 from them into the exchange row x.
+template <typename T, int N>
+__device__ __forceinline__ void rinv_step1(const cplx<T> *sA, const cplx<T> *sB, int n1, const cplx<T> *tw2,
+                                           cplx<T> *x) {
+  constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
+  cplx<T> v[N2];
+  rinv_load<T, N>(sA, sB, n1, v);
   reg_dft<true, N2>(v);
   x[0] = v[0];
 #pragma unroll

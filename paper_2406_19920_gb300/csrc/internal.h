@@ -120,6 +120,8 @@ bool transform_size_supported(int n);
 template <typename T> int plane_modes(int nx, int nz, int *modes);
 // Plane mode used when no tuning result is known.
 template <typename T> int default_plane_mode(int nx, int ny, int nz);
+// The same for the three-field launches of a stage.
+template <typename T> int default_plane_mode_fields(int nx, int ny, int nz);
 // Kernels one forward (or inverse) transform launches: 1 on the plane path, 2 otherwise.
 template <typename T> int transform_launches(const TransformGeom &g);
 

@@ -523,9 +523,10 @@ int ibm_plan_create(int nx, int ny, int nz, int bc, const double h[3], int preci
   // timing and tests)
   p->use_plane = precision == IBM_FP64 ? default_plane_mode<double>(nx, ny, nz) : default_plane_mode<float>(nx, ny, nz);
   p->use_slab = default_use_slab(precision, bc, nx, ny, nz) ? 1 : 0;
-  // three-field solves: split passes (their small CTAs share the SMs
-  // between fields); IBM_PLANE_MODE_FIELDS=m forces another mode
-  p->use_plane_fields = 0;
+  // three-field solves: the default mode for the shape; IBM_PLANE_MODE_FIELDS=m forces
+  // another mode
+  p->use_plane_fields = precision == IBM_FP64 ? default_plane_mode_fields<double>(nx, ny, nz)
+                                              : default_plane_mode_fields<float>(nx, ny, nz);
   if (const char *pm = getenv("IBM_PLANE_MODE_FIELDS")) {
     int modes[8];
     const int n = precision == IBM_FP64 ? plane_modes<double>(nx, nz, modes) : plane_modes<float>(nx, nz, modes);

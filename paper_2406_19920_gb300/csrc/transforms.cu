@@ -157,17 +157,21 @@ template <typename T> int default_plane_mode(int nx, int ny, int nz) {
   // FP32 beyond the planes below.  Measured on GB300 over 40 plane shapes and ny
   // = 8 .. 512 (refined FP32 solve, split passes against plane kernels with the
   // residual in the forward transform, us):
-  //   small planes win by their launches (6 against 11) and at any ny where the
-  //   rows are short: 48x33x24 28.5 / 17, 64x512x64 60 / 53, 128x512x64 80 / 75;
-  //   with long rows up to one CTA an SM: 256x129x32 39 / 32, 256x512x32 77 / 92;
-  //   middle planes from about a third of the SMs on: 96x33x96 30.9 / 31.8,
-  //   96x64x96 33.1 / 31.2, 96x512x96 96 / 87;
-  //   large planes (one CTA an SM) where their CTAs fill one wave of the SMs, or
-  //   two with short rows: 128x64x128 37.7 / 39.2, 128x129x128 54 / 44,
-  //   192x129x96 58 / 47, 192x256x128 128 / 117, 128x512x128 159 / 168,
-  //   256x16x128 33 / 61.
+  //   planes up to 128 x 128 (in place, two CTAs an SM or more) win by their
+  //   launches (6 against 11) and, once they fill the SMs, by bytes:
+  //   48x33x24 28.5 / 20.0, 64x512x64 60 / 51, 96x16x96 29.4 / 29.1, 96x512x96
+  //   96 / 86, 128x128x128 54 / 43, 128x512x128 159 / 133; few large planes do
+  //   not fill the SMs: 128x33x128 33.3 / 38.0, 128x64x128 37.7 / 38.3;
+  //   other small planes at any ny where the rows are short, with long rows up to
+  //   one CTA an SM: 256x129x32 39 / 32, 256x512x32 77 / 92;
+  //   other middle planes from about a third of the SMs on: 192x33x64 33.4 /
+  //   33.3, 64x512x192 138 / 139;
+  //   other large planes (one CTA an SM) where their CTAs fill one wave of the
+  //   SMs, or two with short rows: 192x129x96 58 / 47, 192x256x128 128 / 117,
+  //   192x512x128 243 / 269, 256x16x128 33 / 61.
   if (sizeof(T) == 4 && plane_supported<T>(nx, nz)) {
     const int area = nx * nz;
+    if (nx <= 128 && nz <= 128) return area <= 9216 || ny >= 64;
     const bool wave = (ny >= 80 && ny <= 152) || (nx <= 192 && ny >= 240 && ny <= 304);
     if (area <= 8192) return ny <= 152 || (nx <= 192 && nz <= 256);
     if (area <= 12288) return wave || (nx <= 192 && nz <= 192 && ny >= 56);
@@ -177,6 +181,21 @@ template <typename T> int default_plane_mode(int nx, int ny, int nz) {
 }
 template int default_plane_mode<float>(int, int, int);
 template int default_plane_mode<double>(int, int, int);
+
+template <typename T> int default_plane_mode_fields(int nx, int ny, int nz) {
+  // Three fields a launch.  Measured (one FP32 stage, split passes against plane
+  // kernels, us): 32^3 43.5 / 40.1, 96^3 82 / 78, 128x32x128 73 / 70, 128^3 138 /
+  // 133, 128x256x128 249 / 243, 192x50x96 94 / 88, 192x128x96 154 / 153,
+  // 256x40x32 60 / 57; not 96x128x192 159 / 163, 192x128x128 205 / 213, 256x128x64
+  // 134 / 140, 256x200x32 126 / 131.
+  if (sizeof(T) == 4 && plane_supported<T>(nx, nz)) {
+    if ((nx <= 128 && nz <= 128) || (nx <= 192 && nz <= 96)) return 1;
+    if (nx * nz <= 8192 && 3 * ny <= 152) return 1;
+  }
+  return 0;
+}
+template int default_plane_mode_fields<float>(int, int, int);
+template int default_plane_mode_fields<double>(int, int, int);
 
 bool transform_size_supported(int n) {
 #define X(N) if (n == N) return true;

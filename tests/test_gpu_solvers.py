@@ -457,3 +457,28 @@ def test_residual_pass_marches_every_plane(ny, bc, monkeypatch):
         assert info["rel_residual"] < 1e-3
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("shape", [(128, 17, 128), (128, 9, 8), (8, 9, 128), (96, 9, 128), (128, 9, 96), (12, 10, 96),
+                                   (192, 9, 96), (512, 8, 16), (16, 8, 384)])
+def test_plane_kernels_with_residual_inside(shape, monkeypatch):
+    """FP32 plane kernels, in place up to 128 x 128 and with separate buffers
+    beyond: the refined Poisson solve and the three wall kinds, whose residual
+    is formed inside the forward transform."""
+    monkeypatch.setenv("IBM_PLANE_MODE", "1")
+    nx, ny, nz = shape
+    g = grid(nx, ny, nz)
+    b = synth.white_noise(nx, ny, nz, workload=19, stream=nx).astype(np.float32).astype(np.float64) + 0.25
+    plan = _plan(nx, ny, nz, g, ibm.IBM_FP32_REFINED, 2)
+    try:
+        x = torch.empty(b.shape, dtype=torch.float32, device="cuda")
+        ibm.ibm_poisson_solve(plan, dev(b, torch.float32), x)
+        assert rel_err(host(x), O.poisson_solve(b, g)[0]) <= TOL_FP32
+        for bc in (O.NEUMANN, O.CELL_DIRICHLET, O.FACE_DIRICHLET):
+            bb = b.copy()
+            if bc == O.FACE_DIRICHLET:
+                bb[0] = 0.0
+            ibm.ibm_helmholtz_solve(plan, 0.01, bc, dev(bb, torch.float32), x)
+            assert rel_err(host(x), O.helmholtz_solve(bb, g, 0.01, bc)) <= TOL_FP32, bc
+    finally:
+        ibm.ibm_plan_destroy(plan)
