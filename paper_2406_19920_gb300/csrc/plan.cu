@@ -402,9 +402,30 @@ static int solve_fields_t(ibm_plan_s *p, double c, int nb, const int *field_bc, 
   return IBM_OK;
 }
 
+// The fields one after another through the slab path, in place of one launch
+// per phase for all of them.  Three passes over HBM a field instead of five,
+// and one field's spectrum (101 MB at 384 x 256 x 256) at a time, which L2
+// mostly holds; but nine launches that cannot share the chip.  RK stage with
+// 300 markers, GB300, one launch per phase -> field by field, at nx x 256 x 256:
+// 32 172 -> 192, 64 265 -> 263, 128 493 -> 478, 192 781 -> 751, 256 913 -> 845,
+// 384 1438 -> 1357, 512 2014 -> 1992 us.  So the line lies at nx = 128; where
+// IBM_SLAB=1 forces the slab path, it takes every length.
+static bool slab_fields_apply(const ibm_plan_s *p, int nb, void *const *out, const void *const *addend) {
+  bool in_place = p->use_slab_fields != 0;  // (the slab path's inverse adds in place only)
+  for (int b = 0; b < nb; ++b) in_place &= !addend[b] || addend[b] == out[b];
+  return in_place;
+}
+
 int plan_solve_fields(ibm_plan_s *p, double c, int nb, const int *field_bc, const void *const *in, void *const *out,
                       const void *const *addend, cudaStream_t st) {
   if (nb < 1 || nb > kMaxFields) return set_error(IBM_ERR_ARG, "plan_solve_fields: %d fields", nb);
+  if (slab_fields_apply(p, nb, out, addend)) {
+    for (int b = 0; b < nb; ++b)
+      if (int rc = solve_once_slab(p, pencil_params(p, 1, c, field_bc[b]), static_cast<const float *>(in[b]),
+                                   static_cast<float *>(out[b]), static_cast<const float *>(addend[b]), nullptr, st))
+        return rc;
+    return IBM_OK;
+  }
   for (int b = 0; b + 1 < nb; ++b) {
     if (!p->Sx[b]) {
       cudaError_t e = cudaMalloc(&p->Sx[b], p->nspec * 2 * p->esz);
@@ -527,6 +548,7 @@ int ibm_plan_create(int nx, int ny, int nz, int bc, const double h[3], int preci
   // another mode
   p->use_plane_fields = precision == IBM_FP64 ? default_plane_mode_fields<double>(nx, ny, nz)
                                               : default_plane_mode_fields<float>(nx, ny, nz);
+  p->use_slab_fields = p->use_slab && (nx >= 128 || getenv("IBM_SLAB")) ? 1 : 0;
   if (const char *pm = getenv("IBM_PLANE_MODE_FIELDS")) {
     int modes[8];
     const int n = precision == IBM_FP64 ? plane_modes<double>(nx, nz, modes) : plane_modes<float>(nx, nz, modes);
@@ -539,6 +561,7 @@ int ibm_plan_create(int nx, int ny, int nz, int bc, const double h[3], int preci
                        want, nx, nz);
     }
     p->use_plane_fields = want;
+    p->use_slab_fields = 0;
   }
   if (const char *pm = getenv("IBM_PLANE_MODE")) {
     int modes[8];

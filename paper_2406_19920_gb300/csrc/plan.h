@@ -36,6 +36,7 @@ struct ibm_plan_s {
   int use_plane = 1; // plane mode: 0 split x / z passes; 1 one CTA per plane; C >= 2 a cluster of C CTAs per plane;
                      // -1 (kPlaneDft) tensor-core DFT products (FP32, short planes)
   int use_plane_fields = 0; // plane mode of three-field solves
+  int use_slab_fields = 0;  // a stage's three FP32 fields through the slab path, one after another
   int use_slab = 0;  // FP32 single-field solves through the fused slab path (slab.cu)
   size_t esz;        // element size: 4 or 8
   size_t npts;       // nx * ny * nz

@@ -708,6 +708,13 @@ k_slab(float2 *S, const float2 *__restrict__ twz, const float *__restrict__ lamx
   const int len = rank == Lh ? R - 1 : R;
   const int lr0 = top ? 0 : R - 1, lstep = top ? 1 : -1;  // local row of sweep row u: lr0 + lstep u
   const float sgn = pp.neg_rhs ? -1.f : 1.f;
+  // A face field (j0 = 1; unknowns are rows 1 .. NY - 1, row 0 is the wall
+  // value 0): row 0 takes part as a row of the largest pivot, e_0 = g + 2^60 a,
+  // q_0 = 1 - 2^-60 = 1 in FP32, so row 1 has e_1 = g + a q_0 = g + a, the face
+  // rule's, and the segments stay 32 rows long; its right-hand side is read
+  // as zero and zero is stored.
+  const bool wall_row = pp.j0 != 0 && rank == 0;
+  const float bs = pp.j0 != 0 ? 0x1p60f : (float)pp.beta_s;
   auto rank_of = [](int s2) { return s2 < Lh ? s2 : C - 1 - (s2 - Lh); };
   constexpr uint32_t kHalf = (uint32_t)(R / 2) * NZ * 8;
 
@@ -753,12 +760,13 @@ k_slab(float2 *S, const float2 *__restrict__ twz, const float *__restrict__ lamx
 
     // forward elimination of my segment
     const bool live = !(zm && kz == 0);
-    const float e0 = g + a * (float)(top ? pp.beta_s : pp.beta_e);
+    const float e0 = g + a * (top ? bs : (float)pp.beta_e);
     float ep, D, z;
     const bool cw = __all_sync(0xffffffffu, seg_pivots<float>(a, g, e0, k0, ep, D, z)) && len == R;
     float2 v[R];
 #pragma unroll
     for (int u = 0; u < R; ++u) v[u] = u < len ? slab[(lr0 + lstep * u) * NZ + kz] : make_float2(0.f, 0.f);
+    if (wall_row) v[0] = make_float2(0.f, 0.f);
     float *wc = ws + kz;  // w of sweep row u at wc[NZ u]
     float2 y;
     float prod, qlast;
@@ -866,6 +874,7 @@ k_slab(float2 *S, const float2 *__restrict__ twz, const float *__restrict__ lamx
     if (cw) seg_store<float, R, true, true, NZ>(v, len, wconst, wc, c, live, col, (long)lstep * NZ);
     else seg_store<float, R, false, false, NZ>(v, len, wconst, wc, c, live, col, (long)lstep * NZ);
     if (rank == Lh && live) slab[kz] = xm;
+    if (wall_row) slab[kz] = make_float2(0.f, 0.f);
     if (zm && tid < R) slab[tid * NZ] = make_float2((float)cluster.map_shared_rank(zr, 0)[rank * R + tid], 0.f);
     __syncthreads();
 

@@ -122,54 +122,13 @@ inline ResidualArgs make_args(int nx, int ny, int nz, const StencilCoef &c, cons
   return A;
 }
 
-// r at the four points (x = i0 .. i0 + 3, row k along z, plane j along y) of
-// the wall kind BC, and the compatible right-hand side b - m there (bt, for
-// the norms).  nx % 4 == 0 and 16-byte aligned fields: every row access is
-// a float4; the x neighbours of the four come from the same float4 plus two
-// scalars.
-template <int BC, bool SIGMA>
-__device__ __forceinline__ float4 residual4(const ResidualArgs &A, const float *__restrict__ b,
-                                            const float *__restrict__ x, int j, int k, int i0, float2 m,
-                                            float4 &bt) {
-  const size_t pl = (size_t)A.nx * A.nz;
-  const size_t at = (size_t)j * pl + (size_t)k * A.nx + i0;
-  float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
-  bt = res;
-  if (BC == BC_FACE_DIRICHLET && j == 0) return res;
-  const size_t row = at - i0;
-  const float4 x0 = *reinterpret_cast<const float4 *>(x + at);
-  const float xW = x[row + (i0 == 0 ? A.nx - 1 : i0 - 1)];
-  const float xE = x[row + (i0 + 4 == A.nx ? 0 : i0 + 4)];
-  const long dn = (long)(k + 1 == A.nz ? -(long)(A.nz - 1) * A.nx : (long)A.nx);
-  const long ds = (long)(k == 0 ? (long)(A.nz - 1) * A.nx : -(long)A.nx);
-  const float4 xn = *reinterpret_cast<const float4 *>(x + at + dn);
-  const float4 xs = *reinterpret_cast<const float4 *>(x + at + ds);
-  float4 xd, xu;
-  if (BC == BC_FACE_DIRICHLET) {
-    xd = j - 1 >= 1 ? *reinterpret_cast<const float4 *>(x + at - pl) : make_float4(0.f, 0.f, 0.f, 0.f);
-    xu = j + 1 <= A.ny - 1 ? *reinterpret_cast<const float4 *>(x + at + pl) : make_float4(0.f, 0.f, 0.f, 0.f);
-  } else if (BC == BC_PERIODIC) {
-    xd = *reinterpret_cast<const float4 *>(x + (j > 0 ? at - pl : at + (size_t)(A.ny - 1) * pl));
-    xu = *reinterpret_cast<const float4 *>(x + (j + 1 < A.ny ? at + pl : at - (size_t)(A.ny - 1) * pl));
-  } else {
-    const float gs = BC == BC_NEUMANN ? 1.0f : -1.0f;
-    xd = j > 0 ? *reinterpret_cast<const float4 *>(x + at - pl)
-               : make_float4(gs * x0.x, gs * x0.y, gs * x0.z, gs * x0.w);
-    xu = j + 1 < A.ny ? *reinterpret_cast<const float4 *>(x + at + pl)
-                      : make_float4(gs * x0.x, gs * x0.y, gs * x0.z, gs * x0.w);
-  }
-  const float4 bv = *reinterpret_cast<const float4 *>(b + at);
-  res.x = residual_point<SIGMA>(A, bv.x, m, x0.x, x0.y, xW, xn.x, xs.x, xu.x, xd.x, bt.x);
-  res.y = residual_point<SIGMA>(A, bv.y, m, x0.y, x0.z, x0.x, xn.y, xs.y, xu.y, xd.y, bt.y);
-  res.z = residual_point<SIGMA>(A, bv.z, m, x0.z, x0.w, x0.y, xn.z, xs.z, xu.z, xd.z, bt.z);
-  res.w = residual_point<SIGMA>(A, bv.w, m, x0.w, xE, x0.z, xn.w, xs.w, xu.w, xd.w, bt.w);
-  return res;
-}
-
-// The same four points for a block of consecutive rows of one y plane, with
-// the addressing reduced to 32-bit offsets from the block's first row: xc, bc
-// point at x, b there, xlo / xhi at x one plane below / above (NULL at a wall:
-// the ghost value gs x0), off = (row - first row) nx + i0, k the row's z index.
+// r at the four points x = i0 .. i0 + 3 of a row (z index k) of one y plane,
+// and the compatible right-hand side b - m there (bt, for the norms).  32-bit
+// offsets from the first of the caller's rows: xc, bc point at x, b there, xlo
+// / xhi at x one plane below / above (NULL at a wall: the ghost value gs x0),
+// off = (row - first row) nx + i0.  nx % 4 == 0 and 16-byte aligned fields:
+// every row access is a float4; the x neighbours of the four come from the
+// same float4 plus two scalars.
 template <bool SIGMA>
 __device__ __forceinline__ float4 residual4_ghost(const ResidualArgs &A, float gs, const float *__restrict__ bc,
                                                   const float *__restrict__ xc, const float *__restrict__ xlo,

@@ -842,7 +842,7 @@ int prepare_substep(ibm_plan_s *p, int nmk) {
   int rc = ensure_substep_buffers(p, nmk);
   if (rc) return rc;
   for (int b = 0; b < 2; ++b) {  // the spectra of the stage's three-field Helmholtz launches
-    if (!p->Sx[b]) {
+    if (!p->Sx[b] && !p->use_slab_fields) {
       cudaError_t e = cudaMalloc(&p->Sx[b], p->nspec * 2 * p->esz);
       if (e != cudaSuccess) { p->Sx[b] = nullptr; return cuda_error(e, "field spectrum"); }
       p->bytes += p->nspec * 2 * p->esz;
