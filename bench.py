@@ -65,9 +65,9 @@ N_STATES = 4
 KERNEL_SOURCES = {
     "headline": {"forward": ("slab.cu", "fft2.cuh"), "pencil": ("slab.cu", "seg.cuh", "fft2.cuh"),
                  "inverse": ("slab.cu", "fft2.cuh"), "residual": ("slab.cu", "stencil.cuh", "fft2.cuh")},
-    "stage": {"forward": ("transforms.cu", "axis.cu", "fft2.cuh"),
-              "inverse": ("transforms.cu", "axis.cu", "fft2.cuh"), "pencil": ("pencil.cu", "seg.cuh"),
-              "residual": ("stencil.cu",), "explicit": ("substep.cu",), "divergence": ("substep.cu",),
+    "stage": {"forward": ("transforms.cu", "plane.cuh", "axis.cu", "fft2.cuh", "stencil.cuh"),
+              "inverse": ("transforms.cu", "plane.cuh", "axis.cu", "fft2.cuh"), "pencil": ("pencil.cu", "seg.cuh"),
+              "residual": ("stencil.cu", "stencil.cuh"), "explicit": ("substep.cu",), "divergence": ("substep.cu",),
               "project": ("substep.cu",), "interp": ("ibm_kernels.cu",), "spread": ("ibm_kernels.cu",),
               "motion": ("ibm_kernels.cu",)}}
 # kernel-name prefix -> kind (the names ncu prints)

@@ -42,7 +42,8 @@ struct ibm_plan_s {
   size_t npts;       // nx * ny * nz
   size_t nspec;      // ny * nz * P complex entries
   void *S;           // spectrum workspace
-  void *Sx[2];       // spectra of fields 1 and 2 of a three-field solve (allocated on first use)
+  void *Sx[2];       // spectra of fields 1 and 2 of a three-field solve (allocated on first use; the slab
+                     // path solves field by field in S and needs none)
   void *work;        // real work field (residual / divergence)
   void *bsave;       // copy of an in-place right-hand side
   void *sub[4];      // substep fields du, dv, dw, phi (allocated on first substep)

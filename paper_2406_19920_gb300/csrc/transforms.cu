@@ -12,13 +12,14 @@
 // Z_k = A_k + i B_k from the two Hermitian half spectra.
 //
 // Three kernel families, chosen per plan by its plane mode:
-//   plane kernels   (mode 1, here) one CTA per y-plane: the x transform of
-//                   every row pair lands in a shared-memory plane, the z
+//   plane kernels   (mode 1, plane.cuh) one CTA per y-plane: the x transform
+//                   of every row pair lands in a shared-memory plane, the z
 //                   transform of every column leaves it; one HBM read and
 //                   one write per direction;
 //   axis kernels    (mode 0, axis.cu) x-rows and z-columns in two passes;
 //   cluster kernels (modes 2, 4, 8, cplane.cu) C CTAs per plane.
-// Plane and axis kernels run the two-step register transform of fft2.cuh.
+// Plane and axis kernels run the two-step register transform of fft2.cuh.  This
+// file holds the choice between them.
 #include "plane.cuh"
 
 namespace ibm {
