@@ -73,16 +73,21 @@ template <int N> struct RowT {
   static constexpr size_t smem_f = (size_t)N * 8 + (size_t)N1 * QF * 8;
   static constexpr size_t smem_r = smem_f + (size_t)2 * RP * (N + 8) * 4;  // + the residual tile
   static constexpr size_t a128(size_t b) { return (b + 127) & ~(size_t)127; }
-  // inverse: where each thread has one job in both steps (N1 = N2), the
-  // exchange area lies in the block's own stage (the spectrum is read into
-  // registers before it is written, and it is read before the output rows
-  // are), which lets three CTAs share an SM instead of two
-  static constexpr bool XSTAGE = N1 == N2;
+  // inverse: up to 384 points the exchange area lies in the block's own stage
+  // (the spectrum is read into registers before it is written, and it is read
+  // into registers before the output rows are): three CTAs share an SM instead of
+  // two at 128 to 256 points, two instead of one at 384, where a pass of 384 x 256
+  // x 256 takes 43.6 instead of 57.2 us (one CTA's chain of copies and barriers
+  // left the SM idle).  At 512 two stages alone leave room for one CTA.
+  static constexpr bool XSTAGE = N <= 384;
+  static constexpr int R3 = (RP * N2 + kRowT - 1) / kRowT;  // step-3 jobs a thread (one in step 1)
   static constexpr size_t o_stage = a128((size_t)N * 8 + (XSTAGE ? 0 : (size_t)RP * QI * 8));  // 128-byte aligned tensor-load targets
   static constexpr size_t stage_a = a128(stage_i);
   static constexpr size_t smem_i = o_stage + 2 * stage_a + 16;  // two stages
+  // CTAs an SM the registers are sized for (as many as fit, up to three)
+  static constexpr int CTAS_I = 3 * (smem_i + 1024) <= 233472 ? 3 : 2 * (smem_i + 1024) <= 233472 ? 2 : 1;
   static_assert(!XSTAGE || (size_t)RP * QI * 8 <= stage_a, "the exchange area fits a stage");
-  static_assert(!XSTAGE || RP * N1 == kRowT, "one job per thread in both steps");
+  static_assert(RP * N1 <= kRowT, "one job per thread in step 1");
 };
 
 // Steps of the forward x rows of np row pairs: real rows 2 p and 2 p + 1 at
@@ -429,7 +434,7 @@ k_rows_fwd_res_s(ResidualArgs A, const float *__restrict__ b, const float *__res
 }
 
 template <int N>
-__global__ void __launch_bounds__(kRowT)
+__global__ void __launch_bounds__(kRowT, RowT<N>::CTAS_I)
 k_rows_inv_t(const float2 *__restrict__ S, float *out, bool add, const float2 *__restrict__ tw, int npairs, int rows,
              float scale, const __grid_constant__ CUtensorMap tmap, bool use_tmap, int *err) {
   using Cfg = RowT<N>;
@@ -532,25 +537,32 @@ k_rows_inv_t(const float2 *__restrict__ S, float *out, bool add, const float2 *_
       }
     };
     if constexpr (Cfg::XSTAGE) {
-      // one job per thread: every read of an area ends (barrier) before it
-      // is overwritten: spectrum -> registers -> exchange -> registers -> rows
+      // every read of an area ends (barrier) before it is overwritten:
+      // spectrum -> registers -> exchange -> registers -> rows
       const int job = threadIdx.x;
-      const bool a1 = job < np * N1, a3 = job < np * N2;
+      const bool a1 = job < np * N1;
       const int n1 = job / np, p1 = job - n1 * np;
-      const int p3 = job / N2, k2 = job - p3 * N2;
       float2 v[N2];
       if (a1) step1_load(n1, p1, v);
       __syncthreads();
       if (a1) step1_store(n1, p1, v);
       __syncthreads();
-      float2 u[N1];
-      if (a3) {
+      float2 u[Cfg::R3][N1];
 #pragma unroll
-        for (int q = 0; q < N1; ++q) u[q] = X[p3 * QI + q * N2 + k2];
-        reg_dft<true, N1>(u);
+      for (int r = 0; r < Cfg::R3; ++r) {
+        const int j3 = job + r * kRowT, p3 = j3 / N2, k2 = j3 - p3 * N2;
+        if (j3 < np * N2) {
+#pragma unroll
+          for (int q = 0; q < N1; ++q) u[r][q] = X[p3 * QI + q * N2 + k2];
+          reg_dft<true, N1>(u[r]);
+        }
       }
       __syncthreads();
-      if (a3) step3_store(p3, k2, u);
+#pragma unroll
+      for (int r = 0; r < Cfg::R3; ++r) {
+        const int j3 = job + r * kRowT, p3 = j3 / N2, k2 = j3 - p3 * N2;
+        if (j3 < np * N2) step3_store(p3, k2, u[r]);
+      }
     } else {
       for (int job = threadIdx.x; job < np * N1; job += kRowT) {
         const int n1 = job / np, p = job - n1 * np;
@@ -583,7 +595,7 @@ k_rows_inv_t(const float2 *__restrict__ S, float *out, bool add, const float2 *_
 
 // ---------------------------------------------------------------------------
 // The slab kernel.  Rows y of the slab are the unknowns of every kz pencil
-// (n = ny rows, j0 = 0: Poisson and the cell-centred Helmholtz kinds).  The
+// (n = ny rows; a face field's wall row 0 joins as described at wall_row).  The
 // two-ended sweep splits them as k_pencil_seg does: rows 0 .. m-1 top-down,
 // rows n-1 .. m+1 bottom-up, meeting at m = n/2, in 32-row segments.  CTA r
 // < C/2 owns top segment r (rows 32 r ..), CTA r >= C/2 bottom segment
