@@ -71,7 +71,7 @@ template <int N> struct RowT {
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
   static constexpr size_t stage_i = mx((size_t)P * 2 * RP * 8, (size_t)2 * RP * POUT * 4);
   static constexpr size_t smem_f = (size_t)N * 8 + (size_t)N1 * QF * 8;
-  static constexpr size_t smem_r = smem_f + (size_t)2 * RP * (N + 8) * 4;  // + the residual tile
+  static constexpr size_t smem_r = (size_t)N * 8 + mx((size_t)N1 * QF * 8, (size_t)2 * RP * (N + 8) * 4);  // residual tile, then exchange
   static constexpr size_t a128(size_t b) { return (b + 127) & ~(size_t)127; }
   // inverse: up to 384 points the exchange area lies in the block's own stage
   // (the spectrum is read into registers before it is written, and it is read
@@ -192,7 +192,10 @@ k_rows_fwd_t(const float *__restrict__ in, float2 *__restrict__ S, const float2 
 // pass: the residual r = b - A x (residual4, the slab path's wall kinds) of
 // the CTA's 2 RP rows into a shared tile (pitch N + 8 floats: the two rows a
 // warp reads in step 1 fall on different banks), then the forward x rows of
-// the tile.  r itself never reaches global memory.  norms: the FP64 sums of
+// the tile, whose memory is the exchange area once step 1 has read it into
+// registers: three CTAs an SM to wait for their loads of x instead of two at 384
+// points (384 x 256 x 256 pass 91.8 -> 77.9 us) and one at 512 (refined solve
+// 638 -> 561 us at 512 x 256 x 256).  r itself never reaches global memory.  norms: the FP64 sums of
 // the residual pass, when wanted.
 template <int N, int BC, bool SIGMA>
 __global__ void __launch_bounds__(kRowT)
@@ -202,8 +205,8 @@ k_rows_fwd_res_t(ResidualArgs A, const float *__restrict__ b, const float *__res
   constexpr int TP = N + 8, Q4 = N / 4;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float2 *tw2 = reinterpret_cast<float2 *>(smem_raw);
-  float2 *X = tw2 + N;                                            // [N1][k2][p]
-  float *tile = reinterpret_cast<float *>(X + Cfg::N1 * Cfg::QF);  // [2 RP][TP]
+  float2 *X = tw2 + N;                           // [N1][k2][p]
+  float *tile = reinterpret_cast<float *>(X);  // [2 RP][TP]
   load_step_twiddles<float, N>(tw2, tw);
   pdl_wait();  // x is the predecessor's output
   const int pair0 = blockIdx.x * Cfg::RP;
@@ -230,7 +233,15 @@ k_rows_fwd_res_t(ResidualArgs A, const float *__restrict__ b, const float *__res
   }
   if (norms) block_accumulate(r2, b2, r1, b1, norms);
   __syncthreads();
-  rows_fwd_steps<N>(tile, TP, 1.0f, S, pair0, np, rows, tw2, X);
+  {
+    const int job = threadIdx.x, p = job / Cfg::N1, n1 = job - p * Cfg::N1;
+    float2 v[Cfg::N2];
+    if (job < np * Cfg::N1) rows_fwd_load1<N>(tile, TP, 1.0f, p, n1, v);
+    __syncthreads();
+    if (job < np * Cfg::N1) rows_fwd_store1<N>(X, p, n1, v, tw2);
+  }
+  __syncthreads();
+  rows_fwd_step3<N>(X, S, pair0, np, rows, threadIdx.x, kRowT);
 }
 
 // ---------------------------------------------------------------------------
