@@ -198,3 +198,21 @@ def test_stream_and_block_residual_agree():
     # the same FP32 residual, summed in the same order: both forms agree to
     # the rounding of the correction (about 1e-2 of a 1e-6 correction)
     assert rel_err(streamed, block) <= 1e-7
+
+
+@pytest.mark.parametrize("nx", [8, 32, 64, 128, 192, 512])
+def test_slab_every_row_length(nx):
+    """The x lengths that SLAB_SHAPES leaves out: one or two second-step jobs a
+    thread inside the block's stage (up to 384 points) or beside it (512), and a
+    partial last block (192 points: 21 row pairs a CTA)."""
+    plan, g = _plan((nx, 64, 64), 1)
+    try:
+        b = (synth.white_noise(nx, 64, 64, workload=57, stream=nx) + 0.25).astype(np.float32)
+        ref, _ = O.poisson_solve(b.astype(np.float64), g)
+        rhs = dev(b, torch.float32)
+        phi = torch.empty_like(rhs)
+        ibm.ibm_poisson_solve(plan, rhs, phi)
+        torch.cuda.synchronize()
+        assert rel_err(host(phi), ref) <= TOL_FP32, (nx, rel_err(host(phi), ref))
+    finally:
+        ibm.ibm_plan_destroy(plan)
