@@ -181,8 +181,8 @@ static int dalloc(ibm_plan_s *p, void **ptr, size_t bytes) {
 // ---------------------------------------------------------------------------
 bool default_use_slab(int precision, int bc, int nx, int ny, int nz) {
   // read per plan (A/B timing, tests): IBM_SLAB=0 never, IBM_SLAB=1 wherever the shape is supported, unset
-  // the measured default: 256 x 256 slabs (GB300, refined 256^3 solve 0.317 against 0.332 ms split; at
-  // 128^3 the split passes win, 0.055 against 0.064 ms)
+  // the measured default: 256 x 256 slabs (GB300, refined 256^3 solve 0.229 against 0.288 ms split; at
+  // 128^3 the plane kernels win, 0.041 against 0.064 ms)
   const char *env = getenv("IBM_SLAB");
   if (precision != IBM_FP32_REFINED || bc != IBM_BC_PXZ_WALL_Y || !slab_supported(nx, ny, nz)) return false;
   if (env) return atoi(env) != 0;
