@@ -534,32 +534,34 @@ k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F,
     stencil_origin<T, S>(g, c, X[3 * m], X[3 * m + 1], X[3 * m + 2], bx, by, bz, fx, fy, fz);
     amp = scale * F[t] * dV[m] * (T)g.vol_inv;
   }
-  // bounding box of the CTA's stencil origins
-  int v[6] = {valid ? bx : INT_MAX, valid ? by : INT_MAX, valid ? bz : INT_MAX,
-              valid ? -bx : INT_MAX, valid ? -by : INT_MAX, valid ? -bz : INT_MAX};
+  // bounding box of the CTA's stencil origins; its extent in 64 bits, since the
+  // origin of a marker far outside the box may be any int
+  const int o[3] = {bx, by, bz};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    v[q] = __reduce_min_sync(0xffffffffu, v[q]);
-    if (lane == 0) red[q][warp] = v[q];
+  for (int q = 0; q < 3; ++q) {
+    const int mn = __reduce_min_sync(0xffffffffu, valid ? o[q] : INT_MAX);
+    const int mx = __reduce_max_sync(0xffffffffu, valid ? o[q] : INT_MIN);
+    if (lane == 0) { red[q][warp] = mn; red[q + 3][warp] = mx; }
   }
   __syncthreads();
   int lo[3], dim[3];
-  bool any = false;
+  bool fits = true;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    int mn = INT_MAX, mxn = INT_MAX;
+    int mn = INT_MAX, mx = INT_MIN;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
       mn = min(mn, red[q][w]);
-      mxn = min(mxn, red[q + 3][w]);
+      mx = max(mx, red[q + 3][w]);
     }
-    any = mn != INT_MAX;  // the same for every axis and every thread
-    lo[q] = any ? mn : 0;
-    dim[q] = any ? -mxn - mn + S : 0;  // (max - min) + S points along this axis
+    if (mn > mx) return;  // every entry of the CTA was rejected by the wall rule (the same for every thread)
+    lo[q] = mn;
+    const long d = (long)mx - mn + S;  // points along this axis
+    fits = fits && d <= kSpreadBoxBytes;
+    dim[q] = fits ? (int)d : 0;
   }
-  if (!any) return;  // every entry of the CTA was rejected by the wall rule
   const long vol = (long)dim[0] * dim[1] * dim[2];
-  const bool use_box = vol > 0 && 3 * vol * (long)sizeof(T) <= kSpreadBoxBytes && dim[0] <= g.nx && dim[2] <= g.nz;
+  const bool use_box = fits && 3 * vol * (long)sizeof(T) <= kSpreadBoxBytes && dim[0] <= g.nx && dim[2] <= g.nz;
   T wx[S], wys[S], wz[S];
   delta_weights<T, S>(fx, wx);
   delta_weights<T, S>(fy, wys);

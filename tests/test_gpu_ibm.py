@@ -346,3 +346,30 @@ def test_fp32_spread_lanes_on_points(n, kernel):
             assert rel_err(host(got), want) <= tol
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+def test_fp64_box_spread_with_far_origins():
+    """Pre-aggregated FP64 spreading with a marker more than 2^31 cells outside
+    the periodic box in every CTA, whose stencil origin is the lowest or the
+    highest int: the CTA's box is not formed, its other markers are spread
+    as the oracle has them (the far ones carry no force)."""
+    nx, ny, nz = 48, 40, 32
+    g = grid(nx, ny, nz)
+    n = 45000
+    r = np.random.default_rng(11)
+    X = np.column_stack([3.0 + 0.2 * r.random(n), 1.0 + 0.02 * r.random(n), 2.0 + 0.2 * r.random(n)])
+    F, dV = r.standard_normal((n, 3)), np.full(n, 1e-3)
+    far = np.arange(0, n, 40)
+    fref = O.spread(np.delete(X, far, 0), np.delete(F, far, 0), np.delete(dV, far), g)
+    X[far, 0] = np.where(far % 3 == 0, -1e10, np.where(far % 3 == 1, 1e10, X[far, 0]))
+    X[far, 2] = np.where(far % 3 == 1, X[far, 2], -1e10)
+    F[far] = 0.0
+    plan = ibm.ibm_plan_create(nx, ny, nz, g[3:], ibm.IBM_FP64, 0)
+    try:
+        f = [torch.zeros((ny, nz, nx), dtype=torch.float64, device="cuda") for _ in range(3)]
+        ibm.ibm_spread(plan, n, dev(X, torch.float64), dev(F, torch.float64), dev(dV, torch.float64), *f)
+        torch.cuda.synchronize()
+        for got, ref in zip(f, fref):
+            assert rel_err(host(got), ref) <= TOL_IBM_FP64
+    finally:
+        ibm.ibm_plan_destroy(plan)
