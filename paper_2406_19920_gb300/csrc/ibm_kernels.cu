@@ -103,8 +103,19 @@ __device__ __forceinline__ float third(float x) {
 }
 __device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
 
+// The closed forms hold for a stencil centred on its marker, as every stencil is
+// but for the last bits of f, for FP32 positions so far outside the periodic box
+// that the origin is off by whole points (2^23 cells and more), and for positions
+// that are not finite.  There each point takes the kernel at its own distance: no
+// root of a negative number, and no weight for a point beyond the support or
+// without a distance.
 template <typename T, int S> __device__ __forceinline__ void delta_weights(T f, T (&w)[S]) {
   const T r = f - (T)1;
+  if (!(S == 3 ? fabs(r) <= (T)0.5 : r >= (T)0 && r <= (T)1)) {
+#pragma unroll
+    for (int q = 0; q < S; ++q) w[q] = S == 3 ? phi_roma3<T>(f - (T)q) : phi_peskin4<T>(f - (T)q);
+    return;
+  }
   if constexpr (S == 3) {
     const T s = sqrt(fma((T)-3 * r, r, (T)1));
     const T far = (T)2 - s;

@@ -373,3 +373,50 @@ def test_fp64_box_spread_with_far_origins():
             assert rel_err(host(got), ref) <= TOL_IBM_FP64
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("kernel", [ibm.IBM_DELTA_ROMA3, ibm.IBM_DELTA_PESKIN4])
+@pytest.mark.parametrize("n", [600, 41000])
+@pytest.mark.parametrize("prec", [ibm.IBM_FP64, ibm.IBM_FP32_REFINED])
+def test_markers_without_a_stencil_position(prec, n, kernel):
+    """Markers whose x or z is not a number or infinite have no distance to any
+    point: they read 0 and spread nothing, in each spreading mode, and leave
+    the others' results alone.  Finite positions so far out that FP32 cannot
+    place their stencil get weights of the kernel at some distance: no more
+    than the largest value read, nothing spread by no force."""
+    nx, ny, nz = 48, 40, 32
+    g = grid(nx, ny, nz)
+    dt = torch.float64 if prec == ibm.IBM_FP64 else torch.float32
+    npdt = np.float64 if prec == ibm.IBM_FP64 else np.float32
+    tol = TOL_IBM_FP64 if prec == ibm.IBM_FP64 else TOL_IBM_FP32
+    r = np.random.default_rng(12)
+    X = np.column_stack([6.0 * r.random(n), 0.3 + 1.4 * r.random(n), 6.0 * r.random(n)])
+    F, dV = r.standard_normal((n, 3)), 0.5 + r.random(n)
+    lost, far = np.arange(0, n, 40), np.arange(1, n, 40)
+    X, F, dV = (a.astype(npdt).astype(np.float64) for a in (X, F, dV))
+    u, v, w = (r.standard_normal((ny, nz, nx)).astype(npdt).astype(np.float64) for _ in range(3))
+    v[0] = 0.0
+    keep = np.ones(n, bool)
+    keep[lost] = keep[far] = False
+    Uref = O.interp(X[keep], u, v, w, g, kernel)
+    fref = O.spread(X[keep], F[keep], dV[keep], g, kernel)
+    X[lost, 2 * (lost % 80 > 0)] = np.array([np.nan, np.inf, -np.inf])[np.arange(len(lost)) % 3]
+    X[far, 0] = 1e7 * (1 + np.arange(len(far)))
+    F[far] = 0.0
+    plan = ibm.ibm_plan_create(nx, ny, nz, g[3:], prec, 0)
+    try:
+        ibm.ibm_plan_set_delta(plan, kernel)
+        U = torch.empty((n, 3), dtype=dt, device="cuda")
+        ibm.ibm_interp(plan, n, dev(X, dt), dev(u, dt), dev(v, dt), dev(w, dt), U)
+        Uh = host(U)
+        assert rel_err(Uh[keep], Uref) <= tol
+        assert not Uh[lost].any()
+        assert np.all(np.abs(Uh[far]) <= max(np.abs(a).max() for a in (u, v, w)))
+        for mode in (ibm.IBM_SPREAD_ATOMIC, ibm.IBM_SPREAD_ATOMIC_DIRECT, ibm.IBM_SPREAD_GATHER):
+            ibm.ibm_plan_set_spread(plan, mode)
+            f = [torch.zeros((ny, nz, nx), dtype=dt, device="cuda") for _ in range(3)]
+            ibm.ibm_spread(plan, n, dev(X, dt), dev(F, dt), dev(dV, dt), *f)
+            for got, ref in zip(f, fref):
+                assert rel_err(host(got), ref) <= tol
+    finally:
+        ibm.ibm_plan_destroy(plan)
