@@ -24,6 +24,8 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 #include <mutex>
 
 #include "plan.h"
@@ -36,6 +38,7 @@ struct IbmGrid {
   double inv_h[3];
   float ih_hi[3], ih_lo[3];  // 1/h as float-float for the FP32 path
   double vol_inv;            // 1 / (hx hy hz)
+  unsigned far_x, far_z;     // 2^46 cells along x and z in the working precision (see placed)
   int *err;                  // the plan's error word (flags, rejected-marker count)
 };
 
@@ -51,6 +54,16 @@ template <int S> __device__ __forceinline__ bool clear_of_walls(const IbmGrid &g
   const float lo = fmaf(Y, g.ih_lo[1], p.lo);
   const float r = 0.5f * S;
   return (p.hi - r) + lo >= 0.f && (((float)g.ny - r) - p.hi) - lo >= 0.f;
+}
+// Whether x and z have a place among the periodic points: finite, and less than
+// 2^46 cells away (FP32 takes the fraction of a cell from a float-float).  A marker
+// without one reads 0 and spreads nothing.  On the bits of the magnitude (FP64: of
+// its upper half), since the FP64 kernels are bound by FP64 instructions.
+__device__ __forceinline__ bool placed(const IbmGrid &g, float X, float Z) {
+  return (__float_as_uint(X) & 0x7fffffffu) < g.far_x && (__float_as_uint(Z) & 0x7fffffffu) < g.far_z;
+}
+__device__ __forceinline__ bool placed(const IbmGrid &g, double X, double Z) {
+  return ((unsigned)__double2hiint(X) & 0x7fffffffu) < g.far_x && ((unsigned)__double2hiint(Z) & 0x7fffffffu) < g.far_z;
 }
 __device__ __forceinline__ void report_wall(const IbmGrid &g) {
   atomicOr(g.err, kErrWall);
@@ -103,19 +116,8 @@ __device__ __forceinline__ float third(float x) {
 }
 __device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
 
-// The closed forms hold for a stencil centred on its marker, as every stencil is
-// but for the last bits of f, for FP32 positions so far outside the periodic box
-// that the origin is off by whole points (2^23 cells and more), and for positions
-// that are not finite.  There each point takes the kernel at its own distance: no
-// root of a negative number, and no weight for a point beyond the support or
-// without a distance.
 template <typename T, int S> __device__ __forceinline__ void delta_weights(T f, T (&w)[S]) {
   const T r = f - (T)1;
-  if (!(S == 3 ? fabs(r) <= (T)0.5 : r >= (T)0 && r <= (T)1)) {
-#pragma unroll
-    for (int q = 0; q < S; ++q) w[q] = S == 3 ? phi_roma3<T>(f - (T)q) : phi_peskin4<T>(f - (T)q);
-    return;
-  }
   if constexpr (S == 3) {
     const T s = sqrt(fma((T)-3 * r, r, (T)1));
     const T far = (T)2 - s;
@@ -140,9 +142,10 @@ __device__ __forceinline__ int wrap(int i, int n) {
 // Stencil origin along one axis: s = X/h - o in grid units, first index b
 // and offset f = s - b.  FP64: plain doubles.  FP32: s as a float-float (an
 // error-free product of X with 1/h split into hi + lo, and an error-free
-// sum for the half-cell shift), b from its high part, f = (hi - b) + lo;
-// f is within about 1e-7 grid units of the exact offset, and no FP64
-// instruction is issued (the FP64 pipe is narrow on this part).
+// sum for the half-cell shift), b from its high part and then, where the low part
+// carries s over a point (up to several, 2^23 cells and more outside the periodic
+// box), from the offset itself; f is within about 1e-7 grid units of the exact
+// offset, and no FP64 instruction is issued (the FP64 pipe is narrow on this part).
 template <int S> __device__ __forceinline__ void axis_origin(double X, double ih, float, float, double o, int &b, double &f) {
   const double sx = X * ih - o;
   const double d = (S == 3) ? floor(sx + 0.5) - 1.0 : floor(sx) - 1.0;
@@ -155,8 +158,10 @@ template <int S> __device__ __forceinline__ void axis_origin(float X, double, fl
   const float lo = fmaf(X, ihl, p.lo) + t.lo;
   const float hi = t.hi;
   const float d = (S == 3) ? floorf(hi + 0.5f) - 1.0f : floorf(hi) - 1.0f;
-  b = (int)d;
-  f = (hi - d) + lo;
+  const float e = (hi - d) + lo;
+  const float k = (S == 3) ? floorf(e + 0.5f) - 1.0f : floorf(e) - 1.0f;
+  b = (int)((unsigned)(int)d + (unsigned)(int)k);  // (d + k may have more than 24 bits; wraps, as b + q does, beyond 2^31)
+  f = e - k;
 }
 
 // Component comp's stencil origin (b*) and offsets from it (f*, grid units).
@@ -208,10 +213,11 @@ k_interp(IbmGrid g, int n, const T *X, const T *__restrict__ u, const T *__restr
   }
   const int ml = threadIdx.x - c;  // this marker's first thread in the CTA
   const T mx = X0 ? xs[ml] : X[3 * m], my = X0 ? xs[ml + 1] : X[3 * m + 1], mz = X0 ? xs[ml + 2] : X[3 * m + 2];
-  if (!clear_of_walls<S>(g, my)) {  // the wall rule: no interpolation, no force
-    if (c == 0) report_wall(g);
+  const bool clear = clear_of_walls<S>(g, my);
+  if (!clear || !placed(g, mx, mz)) {  // the wall rule: no interpolation, no force; no place: nothing read
+    if (!clear && c == 0) report_wall(g);
     if (U) U[t] = (T)0;
-    if (F) F[t] = (T)0;
+    if (F) F[t] = clear ? (X0 ? ud_c : Ud[t]) * inv_dt : (T)0;
     return;
   }
   int bx, by, bz;
@@ -261,8 +267,9 @@ k_spread(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, con
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 3 * n) return;
   const int m = t / 3, c = t - 3 * m;
-  if (!clear_of_walls<S>(g, X[3 * m + 1])) {  // the wall rule: not spread
-    if (c == 0) report_wall(g);
+  const bool clear = clear_of_walls<S>(g, X[3 * m + 1]);
+  if (!clear || !placed(g, X[3 * m], X[3 * m + 2])) {  // the wall rule: not spread
+    if (!clear && c == 0) report_wall(g);
     return;
   }
   int bx, by, bz;
@@ -338,8 +345,9 @@ __device__ __forceinline__ unsigned mk_setup(const IbmGrid &g, MkWeights<S> &m, 
   __syncwarp();
   bool ok = false;
   if (lane < nm) {
-    ok = clear_of_walls<S>(g, m.x[3 * lane + 1]);
-    if (!ok) report_wall(g);
+    const bool clear = clear_of_walls<S>(g, m.x[3 * lane + 1]);
+    if (!clear) report_wall(g);
+    ok = clear && placed(g, m.x[3 * lane], m.x[3 * lane + 2]);
   }
   const unsigned okm = __ballot_sync(0xffffffffu, ok);
   const int mk = lane / 6, cb = lane - 6 * mk, ax = cb % 3;
@@ -525,7 +533,7 @@ constexpr int kSpreadBoxMinMarkers = 40000;
 constexpr int kSpreadBoxBytes = 40 * 1024;  // within the default 48 KB limit with the static part
 
 template <typename T, int S>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)  // (at most 64 registers: with three CTAs an SM up to a fifth slower)
 k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F, const T *__restrict__ dV, T *fu,
              T *fv, T *fw, T scale) {
   extern __shared__ __align__(16) unsigned char box_raw[];
@@ -535,9 +543,10 @@ k_spread_box(IbmGrid g, int n, const T *__restrict__ X, const T *__restrict__ F,
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = t < 3 * n ? t / 3 : 0, c = t < 3 * n ? t - 3 * m : 0;
   bool valid = t < 3 * n;
-  if (valid && !clear_of_walls<S>(g, X[3 * m + 1])) {  // the wall rule: not spread
-    if (c == 0) report_wall(g);
-    valid = false;
+  if (valid) {
+    const bool clear = clear_of_walls<S>(g, X[3 * m + 1]);
+    if (!clear && c == 0) report_wall(g);  // the wall rule: not spread
+    valid = clear && placed(g, X[3 * m], X[3 * m + 2]);
   }
   int bx = 0, by = 0, bz = 0;
   T fx = 0, fy = 0, fz = 0, amp = 0;
@@ -716,8 +725,9 @@ k_gather_prep(IbmGrid g, BrickGeom bg, int n, const T *__restrict__ X, const T *
   StencilRec<T> r;
   stencil_origin<T, S>(g, c, X[3 * m], X[3 * m + 1], X[3 * m + 2], r.bx, r.by, r.bz, r.fx, r.fy, r.fz);
   r.amp = scale * F[t] * dV[m] * (T)g.vol_inv;
-  if (!clear_of_walls<S>(g, X[3 * m + 1])) {  // the wall rule: a record that adds nothing
-    if (c == 0) report_wall(g);
+  const bool clear = clear_of_walls<S>(g, X[3 * m + 1]);
+  if (!clear || !placed(g, X[3 * m], X[3 * m + 2])) {  // the wall rule: a record that adds nothing
+    if (!clear && c == 0) report_wall(g);
     r.amp = (T)0;
   }
   const int bx_raw = r.bx, bz_raw = r.bz;
@@ -921,6 +931,20 @@ static IbmGrid ibm_grid(const ibm_plan_s *p) {
     g.ih_lo[d] = (float)(g.inv_h[d] - (double)g.ih_hi[d]);
   }
   g.vol_inv = 1.0 / (p->h[0] * p->h[1] * p->h[2]);
+  auto far = [&](double h) {
+    const double x = std::ldexp(h, 46);
+    if (p->precision == IBM_FP64) {
+      uint64_t u;
+      std::memcpy(&u, &x, sizeof u);
+      return (unsigned)(u >> 32);
+    }
+    const float y = (float)std::min(x, 3e38);
+    unsigned u;
+    std::memcpy(&u, &y, sizeof u);
+    return u;
+  };
+  g.far_x = far(p->h[0]);
+  g.far_z = far(p->h[2]);
   g.err = p->derr;
   return g;
 }
