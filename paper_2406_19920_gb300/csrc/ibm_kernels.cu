@@ -177,22 +177,27 @@ __device__ __forceinline__ void stencil_origin(const IbmGrid &g, int comp, T X, 
 // component (its S^3 accesses independent of each other, so they overlap).
 // With X0 (the substep): the marker's position X = X0 + d and surface
 // velocity Ud = v are formed here (L2), written out, and used at once; the
-// CTA's 32 markers share their coordinates through shared memory.  Without
+// CTA's markers share their coordinates through shared memory.  Without
 // X0 (ibm_interp): X is read.
 // Small CTAs, here and in k_spread, because a body has few warps (FP64, 4,000
 // markers: 375 for 152 SMs) and they should spread over all SMs' pipes: k_interp
-// with 192 -> 96 threads FP64 13.2 -> 11.7 us there, FP32 20,000 markers 9.5 -> 9.1
-// us; k_spread with 256 -> 64 threads FP64 12.5 -> 9.0 us; at 100,000 markers neither
-// changes.
-constexpr int kMarkerThreads = 96;  // a multiple of 3 and of the warp
+// with 192 -> 96 threads FP64 10.7 -> 9.1 us there, FP32 20,000 scattered markers
+// with the 4-point kernel 13.1 -> 11.5 us; k_spread with 256 -> 64 threads FP64 12.3
+// -> 8.8 us.  Large sets fill the SMs either way, and FP32 gathers of scattered markers
+// then run faster from half as many CTAs: 96 -> 192 threads, 3-point kernel 100,000
+// / 124,000 / 300,000 markers 20.9 -> 20.8 / 25.4 -> 24.6 / 56.6 -> 55.3 us, 4-point 41.1 ->
+// 41.0 / 50.1 -> 48.4 / 115.6 -> 111.3 (on a sphere within 1 %); FP64 90.8 -> 94.8 / 112.3
+// -> 111.7 / 262.8 -> 262.4.  The line lies between the first two.
+constexpr int kMarkerThreads = 96, kMarkerThreadsMany = 192;  // multiples of 3 and of the warp
+constexpr int kManyMarkers = 120000;
 constexpr int kSpreadThreads = 64;
 
 template <typename T, int S>
-__global__ void __launch_bounds__(kMarkerThreads)
+__global__ void __launch_bounds__(kMarkerThreadsMany)
 k_interp(IbmGrid g, int n, const T *X, const T *__restrict__ u, const T *__restrict__ v, const T *__restrict__ w,
          const T *__restrict__ du, const T *__restrict__ dv, const T *__restrict__ dw, T *__restrict__ U,
          const T *Ud, T inv_dt, T *__restrict__ F, const T *__restrict__ X0, T *Xout, T *Udout, RigidMotion mo) {
-  __shared__ T xs[kMarkerThreads];
+  __shared__ T xs[kMarkerThreadsMany];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = t / 3, c = t - 3 * m;
   T ud_c = (T)0;
@@ -976,12 +981,12 @@ cudaError_t launch_interp(const ibm_plan_s *p, int n, const T *X, const T *u, co
   if (n <= 0) return cudaSuccess;
   const IbmGrid g = ibm_grid(p);
   const RigidMotion mo = X0 ? rigid_motion(kind, params, t) : RigidMotion{};
-  const int tb = ceil_div(3 * n, kMarkerThreads);
+  const int threads = n < kManyMarkers ? kMarkerThreads : kMarkerThreadsMany, tb = ceil_div(3 * n, threads);
   if (p->delta == IBM_DELTA_PESKIN4)
-    IBM_KTRY(launch_pdl(k_interp<T, 4>, tb, kMarkerThreads, 0, st, g, n, X, u, v, w, du, dv, dw, U, Ud, (T)inv_dt,
+    IBM_KTRY(launch_pdl(k_interp<T, 4>, tb, threads, 0, st, g, n, X, u, v, w, du, dv, dw, U, Ud, (T)inv_dt,
                         F, X0, Xout, Udout, mo));
   else
-    IBM_KTRY(launch_pdl(k_interp<T, 3>, tb, kMarkerThreads, 0, st, g, n, X, u, v, w, du, dv, dw, U, Ud, (T)inv_dt,
+    IBM_KTRY(launch_pdl(k_interp<T, 3>, tb, threads, 0, st, g, n, X, u, v, w, du, dv, dw, U, Ud, (T)inv_dt,
                         F, X0, Xout, Udout, mo));
   return cudaGetLastError();
 }

@@ -422,3 +422,28 @@ def test_markers_without_a_stencil_position(prec, n, kernel):
                 assert rel_err(host(got), ref) <= tol, mode
     finally:
         ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("kernel", [ibm.IBM_DELTA_ROMA3, ibm.IBM_DELTA_PESKIN4])
+@pytest.mark.parametrize("n", [119999, 120000, 120003])
+@pytest.mark.parametrize("prec", [ibm.IBM_FP64, ibm.IBM_FP32_REFINED])
+def test_interp_either_side_of_the_large_ctas(prec, n, kernel):
+    """Interpolation in CTAs of 96 threads, and of 192 from 120,000 markers on (a
+    last CTA partly empty)."""
+    nx, ny, nz = 24, 16, 32
+    g = grid(nx, ny, nz)
+    dt = torch.float64 if prec == ibm.IBM_FP64 else torch.float32
+    npdt = np.float64 if prec == ibm.IBM_FP64 else np.float32
+    r = np.random.default_rng(n)
+    X = np.column_stack([6.28 * r.random(n), 0.3 + 1.4 * r.random(n), 6.28 * r.random(n)]).astype(npdt)
+    u, v, w = (r.standard_normal((ny, nz, nx)).astype(npdt) for _ in range(3))
+    v[0] = 0.0
+    plan = ibm.ibm_plan_create(nx, ny, nz, g[3:], prec, 0)
+    try:
+        ibm.ibm_plan_set_delta(plan, kernel)
+        U = torch.full((n, 3), float("nan"), dtype=dt, device="cuda")
+        ibm.ibm_interp(plan, n, dev(X, dt), dev(u, dt), dev(v, dt), dev(w, dt), U)
+        ref = O.interp(X.astype(np.float64), *(a.astype(np.float64) for a in (u, v, w)), g, kernel)
+        assert rel_err(host(U), ref) <= (TOL_IBM_FP64 if prec == ibm.IBM_FP64 else TOL_IBM_FP32)
+    finally:
+        ibm.ibm_plan_destroy(plan)
