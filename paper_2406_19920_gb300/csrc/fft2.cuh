@@ -94,16 +94,23 @@ template <bool INV, int M, int N, typename C> __device__ __forceinline__ C twidd
   }
 }
 
-// x W_N^M up to a real factor in (0.7, 1]: the product is FACTOR * value.  With
-// the larger of cos and sin taken out, a rotation is two FMAs (t the ratio, at
-// most 1), and the factor goes into the additions that follow.
+// x W_N^M up to a real factor: the product is FACTOR * value.  With the larger of
+// cos and sin taken out, a rotation is two FMAs (t the ratio, at most 1), and the
+// factor goes into the additions that follow.  Of the angles 30 and 60 degrees
+// and their like (the 12-point DFT) the part that is exactly one half is taken out
+// instead, t = sqrt 3: the product of the two rounded constants would stand for
+// the half.
 template <bool INV, int M, int N> struct Rotation {
   static constexpr int m = ((M % N) + N) % N;
   static constexpr ctrig::CS w = ctrig::cs_turn(m, N);
   static constexpr double s = INV ? -w.s : w.s;  // the factor of x is c - i s
-  static constexpr bool by_cos = w.c * w.c >= w.s * w.s;
-  static constexpr double factor = by_cos ? w.c : s;
-  static constexpr double t = by_cos ? s / w.c : w.c / s;
+  static constexpr bool half = (12 * m) % N == 0;  // (not a multiple of a quarter turn: twiddle_const's)
+  static constexpr bool by_cos = (w.c * w.c >= w.s * w.s) != half;
+  static constexpr double part = by_cos ? w.c : s;
+  static constexpr double factor = !half ? part : part > 0 ? 0.5 : -0.5;
+  static constexpr double t = !half                                    ? (by_cos ? s / w.c : w.c / s)
+                              : (part > 0) == ((by_cos ? s : w.c) > 0) ? 1.7320508075688772935
+                                                                       : -1.7320508075688772935;
   template <typename C> static __device__ __forceinline__ C apply(C x) {
     using T = decltype(x.x);
     constexpr T r = (T)t;
@@ -116,7 +123,11 @@ template <bool INV, int M, int N> constexpr bool exact_angle() { return (4 * ((M
 
 // The DFT of (u0, W^k u1, W^2k u2, W^3k u3), W = W_N, with the factors of the
 // rotations folded into the butterflies: 22 FMAs where rotating first takes 28
-// operations.
+// operations.  Against rotating first, the error of a DFT of random numbers is
+// 0.98, 0.97 and 0.95 times as large in FP32 (12, 16 and 32 points), and 0.93, 0.96
+// and 0.98 times in FP64 (with the larger part taken out of every angle the
+// 12-point DFT's was 1.03 times in FP32, and the unrefined 48 x 33 x 24 solve's 4 %
+// larger).
 template <bool INV, int K, int N, typename C> __device__ __forceinline__ void dft4_rotated(C &u0, C &u1, C &u2, C &u3) {
   using T = decltype(u0.x);
   if constexpr (exact_angle<INV, K, N>()) {
@@ -139,18 +150,26 @@ template <bool INV, int K, int N, typename C> __device__ __forceinline__ void df
       t0 = mk<T>(fma(f2, r2.x, u0.x), fma(f2, r2.y, u0.y));
       t1 = mk<T>(fma(-f2, r2.x, u0.x), fma(-f2, r2.y, u0.y));
     }
-    constexpr bool x3 = exact_angle<INV, 3 * K, N>();
-    constexpr T f1 = (T)R1::factor, q = (T)((x3 ? 1.0 : R3::factor) / R1::factor);
+    constexpr T f1 = (T)R1::factor;
     const C r1 = R1::apply(u1);
-    C r3;
-    if constexpr (x3) r3 = twiddle_const<INV, 3 * K, N>(u3);
-    else r3 = R3::apply(u3);
-    const C a = mk<T>(fma(q, r3.x, r1.x), fma(q, r3.y, r1.y));
-    const C b = cmul_mi<INV>(mk<T>(fma(-q, r3.x, r1.x), fma(-q, r3.y, r1.y)));
-    u0 = mk<T>(fma(f1, a.x, t0.x), fma(f1, a.y, t0.y));
-    u2 = mk<T>(fma(-f1, a.x, t0.x), fma(-f1, a.y, t0.y));
-    u1 = mk<T>(fma(f1, b.x, t1.x), fma(f1, b.y, t1.y));
-    u3 = mk<T>(fma(-f1, b.x, t1.x), fma(-f1, b.y, t1.y));
+    if constexpr (exact_angle<INV, 3 * K, N>()) {  // u3 takes part with its exact factor
+      const C r3 = twiddle_const<INV, 3 * K, N>(u3);
+      const C a = mk<T>(fma(f1, r1.x, r3.x), fma(f1, r1.y, r3.y));
+      const C b = cmul_mi<INV>(mk<T>(fma(f1, r1.x, -r3.x), fma(f1, r1.y, -r3.y)));
+      u0 = cadd(t0, a);
+      u2 = csub(t0, a);
+      u1 = cadd(t1, b);
+      u3 = csub(t1, b);
+    } else {
+      constexpr T q = (T)(R3::factor / R1::factor);
+      const C r3 = R3::apply(u3);
+      const C a = mk<T>(fma(q, r3.x, r1.x), fma(q, r3.y, r1.y));
+      const C b = cmul_mi<INV>(mk<T>(fma(-q, r3.x, r1.x), fma(-q, r3.y, r1.y)));
+      u0 = mk<T>(fma(f1, a.x, t0.x), fma(f1, a.y, t0.y));
+      u2 = mk<T>(fma(-f1, a.x, t0.x), fma(-f1, a.y, t0.y));
+      u1 = mk<T>(fma(f1, b.x, t1.x), fma(f1, b.y, t1.y));
+      u3 = mk<T>(fma(-f1, b.x, t1.x), fma(-f1, b.y, t1.y));
+    }
   }
 }
 
