@@ -28,6 +28,7 @@
 
 #include "internal.h"
 #include "seg.cuh"
+#include "sweep.cuh"
 #include "tma.cuh"
 
 namespace ibm {
@@ -41,197 +42,6 @@ __device__ __forceinline__ bool zero_mode_cta(const PencilParams &pp, double *zs
   if (threadIdx.x < 32)
     zero_mode_fp64(pp.zrhs, pp.zsol, zs, pp.ny, pp.inv_ny, pp.hy2, pp.inv_nxnz, mean_out);
   return true;
-}
-
-// Two lanes per pencil, Thomas in excess form from both ends ("twisted"
-// elimination): the even lane eliminates rows 0 .. m-1 top-down, the odd
-// lane rows n-1 .. m+1 bottom-up, and the two meet at row m = n/2, where
-//   (g + a q^T_{m-1} + a q^B_{m+1}) x_m = f_m + a (y^T_{m-1} + y^B_{m+1})
-// (a sum of non-negative terms, like every other pivot).  Each lane then
-// substitutes back towards its end.  The serial depth per pencil is n
-// instead of 2n.  Per row of a half sweep (r = 1/(a + e), w = a r = 1 - q):
-//   forward   y_s = r f_s + w y_{s-1}      (y over f in the shared tile, w kept)
-//   backward  x_s = y_s + w_s x_{s+1}      (straight to the spectrum)
-// The excess of a pencil converges geometrically (all but the longest waves
-// within some 20 to 40 rows), and once it has, the sweep goes on with constant
-// r and w: 4 operations a complex row instead of 11, which is what the FP64
-// sweeps are bound by.  With d the last change of e and w^2 the slope of the
-// map e -> g + a e / (a + e), e is still d w^2 / (1 - w^2) from its fixed
-// point; converged means that this is at most two units in the last place of
-// e, which is what the rounding of the recurrence leaves it moving by (an
-// exact e = e would be missed by pencils that flip between neighbouring
-// values).  The warp looks every kConvRows rows and goes on together.
-// Measured FP64, with the reciprocal of seg.cuh in place of divisions: the
-// streaming sweep of 256 x 128 x 128 74 -> 62 us (the FP64 pipe is busy for 40
-// of them), the tile sweep of 96 x 65 x 64 27 -> 23 us, of the three fields of
-// a stage there 30 -> 18 us.
-constexpr int kConvRows = 8;
-
-template <typename T> __device__ __forceinline__ bool sweep_converged(T e, T en, T w) {
-  constexpr T tol = sizeof(T) == 4 ? (T)0x1p-22 : (T)0x1p-51;
-  const T w2 = w * w;
-  return fabs(en - e) * w2 <= tol * e * ((T)1 - w2);
-}
-
-// One row of the half sweep: y, q and w from the row's e and f; returns the
-// next row's e.
-template <typename T>
-__device__ __forceinline__ T sweep_row(T a, T g, T e, bool neg, cplx<T> f, cplx<T> &y, T &q, T &w, T &rs) {
-  const T r = rcp<T>(a + e);
-  q = e * r;
-  w = a * r;
-  rs = neg ? -r : r;
-  y.x = fma(rs, f.x, w * y.x);
-  y.y = fma(rs, f.y, w * y.y);
-  return fma(a, q, g);
-}
-
-// len: the lane's rows (mlen >= len: the most of any lane of the warp); mask:
-// the warp's lanes that take part.
-template <typename T>
-__device__ __forceinline__ void half_forward(cplx<T> *t, int stp, T *wc, int len, int mlen, T a, T g, T e0, bool neg,
-                                             unsigned mask, cplx<T> &y, T &q) {
-  constexpr int U = kConvRows;
-  T e = e0, w = (T)0, rs = (T)0;
-  y = mk<T>(0, 0);
-  bool conv = false;
-  for (int s0 = 0; s0 < mlen; s0 += U) {
-    const int nu = min(U, len - s0);
-    if (conv) {
-      for (int u = 0; u < nu; ++u, t += stp, wc += stp) {
-        const cplx<T> f = *t;
-        y.x = fma(rs, f.x, w * y.x);
-        y.y = fma(rs, f.y, w * y.y);
-        *t = y;
-        *wc = w;
-      }
-      continue;
-    }
-    bool same = false;
-    if (nu == U) {
-      cplx<T> f[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) f[u] = t[u * stp];
-#pragma unroll
-      for (int u = 0; u < U; ++u, t += stp, wc += stp) {
-        const T en = sweep_row<T>(a, g, e, neg, f[u], y, q, w, rs);
-        if (u == U - 1) same = sweep_converged<T>(e, en, w);
-        e = en;
-        *t = y;
-        *wc = w;
-      }
-    } else {
-      for (int u = 0; u < nu; ++u, t += stp, wc += stp) {
-        e = sweep_row<T>(a, g, e, neg, *t, y, q, w, rs);
-        *t = y;
-        *wc = w;
-      }
-    }
-    conv = __all_sync(mask, same);
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void half_backward(const cplx<T> *t, int stp, const T *wc, int len, cplx<T> x,
-                                              cplx<T> *gcol, long gstep) {
-  t += (len - 1) * stp;
-  wc += (len - 1) * stp;
-  gcol += (len - 1) * gstep;
-#pragma unroll 8
-  for (int s = len; s > 0; --s, t -= stp, wc -= stp, gcol -= gstep) {
-    const cplx<T> y = *t;
-    const T w = *wc;
-    x.x = fma(w, x.x, y.x);
-    x.y = fma(w, x.y, y.y);
-    *gcol = x;
-  }
-}
-
-// Variant for grids with more pencils than the tile kernel keeps resident:
-// no tile; the forward half sweep writes y_s over f_s in the spectrum itself
-// (loads run U to 2U rows ahead of the recurrence), only w stays in shared
-// memory, and the backward sweep reads y_s back (mostly from L2).
-template <typename T> struct SweepDepth { static constexpr int U = 16; };
-template <> struct SweepDepth<double> { static constexpr int U = 8; };
-
-// (Constant rows leave no w in shared memory: kc is the first of them, wk
-// theirs.)
-template <typename T, int U>
-__device__ __forceinline__ void gl_forward(cplx<T> *col, long step, T *wc, int wstep, int len, int mlen, T a, T g,
-                                           T e0, bool neg, unsigned mask, cplx<T> &y, T &q, int &kc, T &wk) {
-  cplx<T> fb[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-    if (u < len) fb[u] = col[u * step];
-  T e = e0, w = (T)0, rs = (T)0;
-  y = mk<T>(0, 0);
-  kc = mlen;
-  for (int s0 = 0; s0 < mlen; s0 += U) {
-    cplx<T> fn[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (s0 + U + u < len) fn[u] = col[(s0 + U + u) * step];
-    if (s0 < kc) {
-      bool same = false;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int s = s0 + u;
-        if (s < len) {
-          const T en = sweep_row<T>(a, g, e, neg, fb[u], y, q, w, rs);
-          if (u == U - 1) same = sweep_converged<T>(e, en, w);
-          e = en;
-          col[s * step] = y;
-          wc[s * wstep] = w;
-        }
-      }
-      if (__all_sync(mask, same)) kc = s0 + U;
-    } else {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int s = s0 + u;
-        if (s < len) {
-          y.x = fma(rs, fb[u].x, w * y.x);
-          y.y = fma(rs, fb[u].y, w * y.y);
-          col[s * step] = y;
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) fb[u] = fn[u];
-  }
-  wk = w;
-}
-
-template <typename T, int U>
-__device__ __forceinline__ void gl_backward(cplx<T> *col, long step, const T *wc, int wstep, int len, int kc, T wk,
-                                            cplx<T> x) {
-  cplx<T> yb[U];
-  T wb[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int s = len - 1 - u;
-    if (s >= 0) { yb[u] = col[s * step]; wb[u] = s < kc ? wc[s * wstep] : wk; }
-  }
-  for (int s0 = len - 1; s0 >= 0; s0 -= U) {
-    cplx<T> yn[U];
-    T wn[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int s = s0 - U - u;
-      if (s >= 0) { yn[u] = col[s * step]; wn[u] = s < kc ? wc[s * wstep] : wk; }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int s = s0 - u;
-      if (s >= 0) {
-        x.x = fma(wb[u], x.x, yb[u].x);
-        x.y = fma(wb[u], x.y, yb[u].y);
-        col[s * step] = x;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) { yb[u] = yn[u]; wb[u] = wn[u]; }
-  }
 }
 
 template <typename T>
@@ -269,7 +79,7 @@ k_pencil_g(Ptr3<cplx<T> *> S_, const T *__restrict__ lamx, const T *__restrict__
   const int wstep = bottom ? -TP : TP;
   const T e0 = g + a * (T)(bottom ? beta_e : beta_s);
   cplx<T> y;
-  T q = (T)0, wk = (T)0;
+  T q = (T)0, wk[2] = {};
   int kc = 0;
   const unsigned mask = __ballot_sync(0xffffffffu, live);
   if (live) gl_forward<T, U>(col, step, wc, wstep, len, m, a, g, e0, pp.neg_rhs != 0, mask, y, q, kc, wk);

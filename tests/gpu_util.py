@@ -88,3 +88,48 @@ class _Scaled(RelErr):
 # gated at twice the L2 tolerance (measured: 2.1e-6 max, 7.8e-7 L2 for 48k
 # markers at 96x64x96).
 IBM_INF_RATIO = 2.0
+
+
+def solve_extended(b, h, c=None, field_bc=0):
+    """x of L x = b (c None: wall-bounded Poisson, zero-mean b and x) or of
+    (I - c L) x = b for a wall kind, in extended precision (numpy longdouble):
+    FFTs in x and z, then per pencil the elimination of tridiag(-a, 2 a + g, -a)
+    with the pivots' excess e = pivot - a carried as such (e' = g + a e / (a + e)),
+    whose terms are all positive.  Its error stays below 1e-16 where the FP64
+    oracle's grows with the condition number (1e-12 at 511 rows, c = 50).
+    field_bc: 0 cell Neumann, 1 cell Dirichlet, 2 face Dirichlet (plane 0 of x is 0)."""
+    ld = np.longdouble
+    ny, nz, nx = b.shape
+    f = np.fft.fft(np.fft.rfft(np.asarray(b, dtype=ld), axis=2), axis=1)
+    assert f.dtype == np.clongdouble
+
+    def lam(n, m, step):
+        s = np.sin(4 * np.arctan(ld(1)) * np.arange(m).astype(ld) / n)
+        return 4 * s * s / ld(step) ** 2
+
+    lz, lx = lam(nz, nz, h[2]), lam(nx, nx // 2 + 1, h[0])
+    lam_xz = lz[:, None] + lx[None, :]
+    hy2 = ld(h[1]) ** 2
+    if c is None:
+        a, g, f, beta, j0 = 1 / hy2, lam_xz.copy(), -f, 0, 0
+        g[0, 0] = 1  # the singular pencil is solved below
+    else:
+        a, g, beta, j0 = ld(c) / hy2, 1 + ld(c) * lam_xz, (0, 2, 1)[field_bc], int(field_bc == 2)
+    n = ny - j0
+    y, w = np.empty((n,) + g.shape, np.clongdouble), np.empty((n,) + g.shape, ld)
+    e = g + a * beta
+    for k in range(n):
+        r = 1 / (a + e if k < n - 1 else e + a * beta)
+        w[k] = a * r
+        y[k] = r * f[j0 + k] + (w[k] * y[k - 1] if k else 0)
+        e = g + a * (e * r)
+    for k in range(n - 2, -1, -1):
+        y[k] += w[k] * y[k + 1]
+    if c is None:
+        m = -f[:, 0, 0].real
+        m = m - m.mean()
+        z = np.concatenate([[ld(0)], hy2 * np.cumsum(np.cumsum(m)[:-1])])
+        y[:, 0, 0] = z - z.mean()
+    x = np.zeros_like(f)
+    x[j0:] = y
+    return np.fft.irfft(np.fft.ifft(x, axis=1), n=nx, axis=2)
