@@ -66,8 +66,12 @@ template <typename T> struct F3 {
 //   YZ(j, k) = (v_{k-1} + v_k)(w_{j-1} + w_j)
 // (times 4, on the cell edges) one flux serves the two components it
 // transports, and the y and z neighbours' fluxes are the thread's own but at
-// the ends.  That leaves 82 operations a point (111 with every flux formed
-// where it is used) and 16 shared-memory loads (40).
+// the ends.  That leaves some 80 operations a point (111 with every flux formed
+// where it is used) and 16 shared-memory loads (40).  Every difference of two
+// fluxes is one FMA on the second one's factors, with the first one's rounded
+// product, and the y term, the largest between walls, is the last one added,
+// unrounded: with two rounded products and the sum in another order N_v loses 4 % of
+// its accuracy in FP32.
 // Wall rules in y: u, w cell-centred with the no-slip ghost (-value) in the
 // Laplacian and zero wall flux in the advective y-flux; v on faces, zero at
 // the walls (j = 0 stored as the wall, j = ny not stored).
@@ -187,18 +191,21 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
   for (int z = 0; z < 4; ++z) vc[z] = V[(z - 1) * PI];
 #pragma unroll
   for (int z = 0; z < 3; ++z) w0[z] = W[z * PI];
-  // fluxes on the lower edges of plane j (zero at the wall j = 0)
-  T xy[2] = {}, xyE[2] = {}, yz[3] = {}, yy[2] = {};
+  // fluxes XY, YZ on the lower edges of plane j (zero at the wall j = 0), their differences to the next edge along x
+  // and z, and twice the average of v under the plane
+  T xy[2] = {}, dxy[2] = {}, yz[2] = {}, dyz[2] = {}, va[2] = {};
   if (jb > 0) {
+    T A[3], B[3];
+#pragma unroll
+    for (int z = 0; z < 3; ++z) { A[z] = vc[z] + vc[z + 1]; B[z] = wd[z] + w0[z]; }
 #pragma unroll
     for (int z = 0; z < 2; ++z) {
       xy[z] = (vW[z] + vc[z + 1]) * (ud[z] + u0[z]);
-      xyE[z] = (vc[z + 1] + vE[z]) * (uEd[z] + uE[z]);
-      const T a = vd[z] + vc[z + 1];
-      yy[z] = a * a;
+      dxy[z] = fma(vc[z + 1] + vE[z], uEd[z] + uE[z], -xy[z]);
+      yz[z] = A[z] * B[z];
+      dyz[z] = fma(A[z + 1], B[z + 1], -yz[z]);
+      va[z] = vd[z] + vc[z + 1];
     }
-#pragma unroll
-    for (int z = 0; z < 3; ++z) yz[z] = (vc[z] + vc[z + 1]) * (wd[z] + w0[z]);
   }
   const bool n_prev = cf.zet != (T)0;  // N^{n-2} unused (and maybe unset) at stage 1
   int ps = 0;                          // p slot of plane j
@@ -232,7 +239,8 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
     for (int z = 0; z < 2; ++z) { nu[z] = nuN[z]; nv[z] = nvN[z]; nw[z] = nwN[z]; }
     if (j + 1 < je) fetch_n(at + plane);
     // plane j + 1 and the fluxes on the upper edges
-    T u1[2], uE1[2], vc1[4], vW1[2], vE1[2], w1[3], xy1[2], xyE1[2], yz1[3], yy1[2], uu[2], wu[2], vu[2];
+    T u1[2], uE1[2], vc1[4], vW1[2], vE1[2], w1[3], xy1[2], dxy1[2], yz1[2], dyz1[2], uu[2], wu[2], vu[2];
+    T xyj[2], yzj[2];  // differences of XY, YZ along y
     if (!hi) {
       const T *U1 = su + s1 + c, *V1 = sv + s1 + c, *W1 = sw + s1 + c;
 #pragma unroll
@@ -246,21 +254,29 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
       for (int z = 0; z < 4; ++z) vc1[z] = V1[(z - 1) * PI];
 #pragma unroll
       for (int z = 0; z < 3; ++z) w1[z] = W1[z * PI];
+      T A[3], B[3];
+#pragma unroll
+      for (int z = 0; z < 3; ++z) { A[z] = vc1[z] + vc1[z + 1]; B[z] = w0[z] + w1[z]; }
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        xy1[z] = (vW1[z] + vc1[z + 1]) * (u0[z] + u1[z]);
-        xyE1[z] = (vc1[z + 1] + vE1[z]) * (uE[z] + uE1[z]);
+        const T a = vW1[z] + vc1[z + 1], b = u0[z] + u1[z];
+        xy1[z] = a * b;
+        xyj[z] = fma(a, b, -xy[z]);
+        dxy1[z] = fma(vc1[z + 1] + vE1[z], uE[z] + uE1[z], -xy1[z]);
+        yz1[z] = A[z] * B[z];
+        yzj[z] = fma(A[z], B[z], -yz[z]);
+        dyz1[z] = fma(A[z + 1], B[z + 1], -yz1[z]);
         uu[z] = u1[z];
         wu[z] = w1[z];
         vu[z] = vc1[z + 1];
       }
-#pragma unroll
-      for (int z = 0; z < 3; ++z) yz1[z] = (vc1[z] + vc1[z + 1]) * (w0[z] + w1[z]);
     } else {
       // the wall above: no plane, no flux; IO: the outlet's values
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        u1[z] = uE1[z] = vW1[z] = vE1[z] = xy1[z] = xyE1[z] = (T)0;
+        u1[z] = uE1[z] = vW1[z] = vE1[z] = xy1[z] = dxy1[z] = yz1[z] = dyz1[z] = (T)0;
+        xyj[z] = -xy[z];
+        yzj[z] = -yz[z];
         uu[z] = -u0[z];
         wu[z] = -w0[z];
         vu[z] = (T)0;
@@ -268,7 +284,7 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
 #pragma unroll
       for (int z = 0; z < 4; ++z) vc1[z] = (T)0;
 #pragma unroll
-      for (int z = 0; z < 3; ++z) w1[z] = yz1[z] = (T)0;
+      for (int z = 0; z < 3; ++z) w1[z] = (T)0;
       if (IO && inside) {
 #pragma unroll
         for (int z = 0; z < 2; ++z) {
@@ -277,17 +293,12 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
           uu[z] = 2 * ug - u0[z];
           wu[z] = 2 * wg - w0[z];
           vu[z] = vg;
-          xy1[z] = (vo[kz * nx + iw] + vg) * (ug + ug);
-          yz1[z] = (vo[ks * nx + i] + vg) * (wg + wg);
+          xyj[z] = fma(vo[kz * nx + iw] + vg, ug + ug, -xy[z]);
+          yzj[z] = fma(vo[ks * nx + i] + vg, wg + wg, -yz[z]);
         }
       }
     }
     const T vb[2] = {lo ? v_wall : vc[1], lo ? v_wall : vc[2]};
-#pragma unroll
-    for (int z = 0; z < 2; ++z) {
-      const T a = vb[z] + vu[z];
-      yy1[z] = a * a;
-    }
     // the rest of plane j
     U = su + s0 + c; V = sv + s0 + c; W = sw + s0 + c;
     const T *Pp = sp + ps + c;
@@ -296,13 +307,13 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
     const T wk[4] = {wS, w0[0], w0[1], w0[2]};  // w at k - 1 .. k + 2
     const T uEk[3] = {uES, uE[0], uE[1]};       // u at i + 1, k - 1 .. k + 1
     const T pS = Pp[-PI];
-    T wW[3], xz[3], zz[3], p0[2];
+    T wW[3], xzA[3], xzB[3], wa[3], p0[2];
 #pragma unroll
     for (int z = 0; z < 3; ++z) {
       wW[z] = W[z * PI - 1];
-      xz[z] = (wW[z] + w0[z]) * (uk[z] + uk[z + 1]);
-      const T a = wk[z] + wk[z + 1];
-      zz[z] = a * a;
+      xzA[z] = wW[z] + w0[z];
+      xzB[z] = uk[z] + uk[z + 1];
+      wa[z] = wk[z] + wk[z + 1];
     }
 #pragma unroll
     for (int z = 0; z < 2; ++z) p0[z] = Pp[z * PI];
@@ -310,10 +321,11 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
     for (int z = 0; z < 2; ++z) {
       const size_t o = at + (size_t)z * nx;
       const T uw = U[z * PI - 1], wE = W[z * PI + 1];
+      const T xz = xzA[z] * xzB[z], va1 = vb[z] + vu[z];
       // u (x-faces)
       {
         const T a = u0[z] + uE[z], b = uw + u0[z];  // twice the averages
-        const T N = (a * a - b * b) * cf.qx + (xy1[z] - xy[z]) * cf.qy + (xz[z + 1] - xz[z]) * cf.qz;
+        const T N = fma(xyj[z], cf.qy, fma(fma(a, a, -(b * b)), cf.qx, fma(xzA[z + 1], xzB[z + 1], -xz) * cf.qz));
         const T lx = uE[z] - 2 * u0[z] + uw, lz = uk[z + 2] - 2 * u0[z] + uk[z];
         const T ly = uu[z] - 2 * u0[z] + (lo ? -u0[z] : ud[z]);
         if (inside) {
@@ -323,8 +335,8 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
       }
       // w (z-faces)
       {
-        const T xzE = (w0[z] + wE) * (uEk[z] + uEk[z + 1]);
-        const T N = (zz[z + 1] - zz[z]) * cf.qz + (xzE - xz[z]) * cf.qx + (yz1[z] - yz[z]) * cf.qy;
+        const T N = fma(yzj[z], cf.qy, fma(fma(wa[z + 1], wa[z + 1], -(wa[z] * wa[z])), cf.qz,
+                                           fma(w0[z] + wE, uEk[z] + uEk[z + 1], -xz) * cf.qx));
         const T lx = wE - 2 * w0[z] + wW[z], lz = wk[z + 2] - 2 * w0[z] + wk[z];
         const T ly = wu[z] - 2 * w0[z] + (lo ? -w0[z] : wd[z]);
         if (inside) {
@@ -336,7 +348,7 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
       // v (y-faces, interior j = 1 .. ny - 1)
       {
         const T v0 = vc[z + 1];
-        const T N = (yy1[z] - yy[z]) * cf.qy + (xyE[z] - xy[z]) * cf.qx + (yz[z + 1] - yz[z]) * cf.qz;
+        const T N = fma(fma(va1, va1, -(va[z] * va[z])), cf.qy, fma(dxy[z], cf.qx, dyz[z] * cf.qz));
         const T lx = vE[z] - 2 * v0 + vW[z], lz = vc[z + 2] - 2 * v0 + vc[z];
         const T ly = vu[z] - 2 * v0 + vd[z];
         if (inside) {
@@ -345,19 +357,20 @@ k_explicit(int nx, int ny, int nz, int jc, const T *__restrict__ u_, const T *__
           Nv[o] = lo ? (T)0 : N;
         }
       }
+      va[z] = va1;
     }
     // plane j becomes plane j - 1
 #pragma unroll
     for (int z = 0; z < 2; ++z) {
       ud[z] = u0[z]; u0[z] = u1[z]; uE[z] = uE1[z];
       vd[z] = vb[z]; vW[z] = vW1[z]; vE[z] = vE1[z];
-      xy[z] = xy1[z]; xyE[z] = xyE1[z]; yy[z] = yy1[z];
+      xy[z] = xy1[z]; dxy[z] = dxy1[z]; yz[z] = yz1[z]; dyz[z] = dyz1[z];
       pd[z] = p0[z];
     }
 #pragma unroll
     for (int z = 0; z < 4; ++z) vc[z] = vc1[z];
 #pragma unroll
-    for (int z = 0; z < 3; ++z) { wd[z] = w0[z]; w0[z] = w1[z]; yz[z] = yz1[z]; }
+    for (int z = 0; z < 3; ++z) { wd[z] = w0[z]; w0[z] = w1[z]; }
     const int t = s0;
     s0 = s1; s1 = s2; s2 = s3; s3 = t;
     ps = ps == 2 * PL ? 0 : ps + PL;
