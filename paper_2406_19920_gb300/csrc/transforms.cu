@@ -20,6 +20,9 @@
 //   cluster kernels (modes 2, 4, 8, cplane.cu) C CTAs per plane.
 // Plane and axis kernels run the two-step register transform of fft2.cuh.  This
 // file holds the choice between them.
+#include <algorithm>
+#include <mutex>
+
 #include "plane.cuh"
 
 namespace ibm {
@@ -153,30 +156,59 @@ template <typename T> int plane_modes(int nx, int nz, int *modes) {
 template int plane_modes<float>(int, int, int *);
 template int plane_modes<double>(int, int, int *);
 
+static int sm_count() {
+  static std::once_flag once;
+  static int sms = 0;
+  std::call_once(once, [] {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 0;
+  });
+  return std::max(sms, 1);  // (without a device the plan is refused later)
+}
+
+// The last wave of n CTAs, one an SM, fills more than a third of the SMs.
+static bool last_wave_filled(int n, int sms) {
+  const int last = n % sms;
+  return last == 0 || 20 * last >= 7 * sms;
+}
+
 template <typename T> int default_plane_mode(int nx, int ny, int nz) {
   // FP64 (arithmetic-bound) takes the split passes at every size, and so does
-  // FP32 beyond the planes below.  Measured on GB300 over 40 plane shapes and ny
-  // = 8 .. 512 (refined FP32 solve, split passes against plane kernels with the
-  // residual in the forward transform, us):
+  // FP32 beyond the planes below.  The lines follow refined FP32 Poisson and
+  // Helmholtz solves timed on GB300 (152 SMs) for every plane shape at 28 ny from 8
+  // to 512, split passes against plane kernels with the residual in the forward
+  // transform (us, Poisson):
   //   planes up to 128 x 128 (in place, two CTAs an SM or more) win by their
-  //   launches (6 against 11) and, once they fill the SMs, by bytes:
-  //   48x33x24 28.5 / 20.0, 64x512x64 60 / 51, 96x16x96 29.4 / 29.1, 96x512x96
-  //   96 / 86, 128x128x128 54 / 43, 128x512x128 159 / 133; few large planes do
-  //   not fill the SMs: 128x33x128 33.3 / 38.0, 128x64x128 37.7 / 38.3;
-  //   other small planes at any ny where the rows are short, with long rows up to
-  //   one CTA an SM: 256x129x32 39 / 32, 256x512x32 77 / 92;
-  //   other middle planes from about a third of the SMs on: 192x33x64 33.4 /
-  //   33.3, 64x512x192 138 / 139;
-  //   other large planes (one CTA an SM) where their CTAs fill one wave of the
-  //   SMs, or two with short rows: 192x129x96 58 / 47, 192x256x128 128 / 117,
-  //   192x512x128 243 / 269, 256x16x128 33 / 61.
+  //   launches (6 against 11) and, once they fill the SMs, by bytes: 48x33x24
+  //   30.3 / 21.1, 96x16x96 30.5 / 29.9, 96x512x96 96.2 / 86.3, 128x80x128
+  //   44.9 / 39.7, 128x512x128 153.5 / 133.0; not the few large planes that
+  //   leave SMs idle: 128x33x128 34.0 / 38.6, 128x64x128 37.5 / 38.7,
+  //   96x33x128 33.1 / 35.5;
+  //   other small planes at any ny where the rows are short, with long rows up
+  //   to one CTA an SM: 192x512x32 74.6 / 68.0, 256x128x32 38.0 / 31.0,
+  //   256x512x32 77.4 / 91.6;
+  //   other middle planes from about a third of the SMs on, and beyond one
+  //   wave where the last one is not nearly empty: 48x56x192 39.5 / 33.9,
+  //   64x153x192 57.0 / 63.8, 64x228x192 69.2 / 70.8, 64x256x192 71.4 / 69.2,
+  //   64x305x192 90.1 / 96.9; 192x153x48 49.5 / 47.1 (short columns) and its
+  //   like at every ny;
+  //   other large planes (one CTA an SM) where their CTAs fill most of one
+  //   wave, or of two with short rows: 192x80x96 46.0 / 43.5, 96x80x256 55.9 /
+  //   59.6, 96x100x256 64.9 / 62.4, 256x100x96 55.0 / 59.2, 256x128x96 62.5 /
+  //   59.7, 192x256x128 126.8 / 115.6, 192x512x128 241.4 / 266.6.
   if (sizeof(T) == 4 && plane_supported<T>(nx, nz)) {
-    const int area = nx * nz;
-    if (nx <= 128 && nz <= 128) return area <= 9216 || ny >= 64;
-    const bool wave = (ny >= 80 && ny <= 152) || (nx <= 192 && ny >= 240 && ny <= 304);
-    if (area <= 8192) return ny <= 152 || (nx <= 192 && nz <= 256);
-    if (area <= 12288) return wave || (nx <= 192 && nz <= 192 && ny >= 56);
-    if (area <= kPlaneArea) return wave;
+    const int area = nx * nz, sms = sm_count();
+    const bool one = ny <= sms;                                             // one wave
+    const bool two = nx <= 192 && 19 * ny >= 30 * sms && ny <= 2 * sms;     // most of two
+    if (nx <= 128 && nz <= 128) return area <= 9216 || (area <= 12288 ? 5 : 4) * ny >= 2 * sms;
+    if (area <= 8192) return one || (nx <= 192 && nz <= 256);
+    if (area <= 12288 && nx <= 192 && nz <= 192)
+      return 11 * ny >= 4 * sms && (one || nz <= 48 || last_wave_filled(ny, sms));
+    if (area <= kPlaneArea) {
+      const bool most = area <= 18432 ? 19 * ny >= 10 * sms : nx <= 192 ? 9 * ny >= 5 * sms : 11 * ny >= 8 * sms;
+      return (one && most) || two;
+    }
   }
   return 0;
 }
@@ -184,14 +216,19 @@ template int default_plane_mode<float>(int, int, int);
 template int default_plane_mode<double>(int, int, int);
 
 template <typename T> int default_plane_mode_fields(int nx, int ny, int nz) {
-  // Three fields a launch.  Measured (one FP32 stage, split passes against plane
-  // kernels, us): 32^3 43.5 / 40.1, 96^3 82 / 78, 128x32x128 73 / 70, 128^3 138 /
-  // 133, 128x256x128 249 / 243, 192x50x96 94 / 88, 192x128x96 154 / 153,
-  // 256x40x32 60 / 57; not 96x128x192 159 / 163, 192x128x128 205 / 213, 256x128x64
-  // 134 / 140, 256x200x32 126 / 131.
+  // Three fields a launch.  Measured on GB300 for every plane shape up to 24,576
+  // points at 19 ny from 8 to 512 (one FP32 stage, plane kernels over split
+  // passes): planes up to 96 x 96 and 192 x 48 0.8 to 0.99 at any ny; 128 x 128
+  // 1.05, 1.02, 1.01 at ny = 8, 16, 24, 0.90 to 1.0 from 33 on; 192 x 96, one CTA an
+  // SM, by the last wave of its 3 ny CTAs: 0.92 at ny = 50 (150 CTAs), 1.06 at 56,
+  // 1.00 at 80, 0.95 at 100, 1.03 at 256 (768 CTAs), 0.99 at 304; other small planes
+  // up to one wave: 256 x 32 0.92 at 50, 1.03 at 56; not 96 x 192 (1.03 at 128), 192 x
+  // 128 (1.04), 256 x 64 (1.06).
   if (sizeof(T) == 4 && plane_supported<T>(nx, nz)) {
-    if ((nx <= 128 && nz <= 128) || (nx <= 192 && nz <= 96)) return 1;
-    if (nx * nz <= 8192 && 3 * ny <= 152) return 1;
+    const int area = nx * nz, sms = sm_count(), ctas = 3 * ny;
+    if (nx <= 128 && nz <= 128) return area <= 9216 || 20 * ctas >= 9 * sms;
+    if (nx <= 192 && nz <= 96) return area <= 9216 || last_wave_filled(ctas, sms);
+    if (area <= 8192) return ctas <= sms;
   }
   return 0;
 }
