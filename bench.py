@@ -66,7 +66,7 @@ KERNEL_SOURCES = {
     "headline": {"forward": ("slab.cu", "fft2.cuh"), "pencil": ("slab.cu", "seg.cuh", "fft2.cuh"),
                  "inverse": ("slab.cu", "fft2.cuh"), "residual": ("slab.cu", "stencil.cuh", "fft2.cuh")},
     "stage": {"forward": ("transforms.cu", "plane.cuh", "axis.cu", "fft2.cuh", "stencil.cuh"),
-              "inverse": ("transforms.cu", "plane.cuh", "axis.cu", "fft2.cuh"), "pencil": ("pencil.cu", "seg.cuh"),
+              "inverse": ("transforms.cu", "plane.cuh", "axis.cu", "fft2.cuh"), "pencil": ("pencil.cu", "seg.cuh", "sweep.cuh"),
               "residual": ("stencil.cu", "stencil.cuh"), "explicit": ("substep.cu",), "divergence": ("substep.cu",),
               "project": ("substep.cu",), "interp": ("ibm_kernels.cu",), "spread": ("ibm_kernels.cu",),
               "motion": ("ibm_kernels.cu",)}}
@@ -246,8 +246,9 @@ def solve_kind_bytes(n, esz=4, refine=HEAD_REFINE, fused=True):
     forward: read field + write spectrum per transform; pencil: read + write
     spectrum; inverse: read spectrum + write field, plus the read of the
     field the correction is added to; residual: read b and x, write r, or,
-    `fused` (the slab path), read b and x and write the correction's
-    spectrum (its forward x rows run in the same pass).  The spectrum round
+    `fused` (the slab path and the plane kernels), read b and x and write the
+    correction's spectrum (its forward transform, or the x rows of it, runs in
+    the same pass).  The spectrum round
     trip between split x and z passes is not counted (it is not compulsory:
     a plane kernel avoids it)."""
     pts = n ** 3
@@ -272,29 +273,41 @@ def slab_path(n, precision_fp32, bc=None, env=None):
     return n == 256
 
 
+def fused_residual(n, precision_fp32, bc=None, env=None):
+    """Whether an n^3 plan forms the refinement residual inside the
+    correction's forward transform: the slab path, and the FP32 plane kernels
+    (the library's default for cubes up to 128^3, wall-bounded or triply
+    periodic; IBM_PLANE_MODE forces them on or off)."""
+    if not precision_fp32:
+        return False
+    if slab_path(n, precision_fp32, bc, env):
+        return True
+    mode = (env or {}).get("IBM_PLANE_MODE", os.environ.get("IBM_PLANE_MODE"))
+    return mode == "1" if mode is not None else n <= 128
+
+
 def algorithmic_bytes(kind, esz=4):
     """Compulsory HBM bytes per step of the 128^3 RK-stage extra, per kernel kind.
 
     pts = nx ny nz real points; spec = ny nz (nx/2+1) complex entries.  A
     stage transforms five fields each way: the three Helmholtz increments
     (one shared launch set) and the Poisson solve plus its refinement.
-    forward: read field + write spectrum, x5; inverse: read spectrum + write
-    field, x5, plus the added field of the three Helmholtz increments and of
-    the refinement update; pencil: read + write spectrum, x5; residual: read
-    b, x, write r; explicit: read u,v,w,p, N x3, write du,dv,dw, N x3;
-    divergence: read u,v,w, write b; project: read u,v,w,p,phi, write
+    forward: read field + write spectrum, x4; residual (the fifth forward
+    transform, with the residual formed inside it): read b, x, write
+    spectrum; inverse: read spectrum + write field, x5, plus the added field
+    of the three Helmholtz increments and of the refinement update; pencil:
+    read + write spectrum, x5; explicit: read u,v,w,p, N x3, write du,dv,dw,
+    N x3; divergence: read u,v,w, write b; project: read u,v,w,p,phi, write
     u,v,w,p; markers: positions, weights, 27-point stencils of 3 components.
-    The spectrum round trip between the split x and z passes is not counted
-    (it is not compulsory: the one-CTA plane kernels avoid it).
     """
     pts = NX * NY * NZ
     spec = NY * NZ * (NX // 2 + 1)
     cs = 2 * esz
     table = {
-        "forward": 5 * (pts * esz + spec * cs),
+        "forward": 4 * (pts * esz + spec * cs),
         "inverse": 5 * (spec * cs + pts * esz) + 4 * pts * esz,
         "pencil": 5 * 2 * spec * cs,
-        "residual": 3 * pts * esz,
+        "residual": 2 * pts * esz + spec * cs,
         "explicit": 13 * pts * esz,
         "divergence": 4 * pts * esz,
         "project": 9 * pts * esz,
@@ -315,6 +328,24 @@ def kernel_kind(name):
     return None
 
 
+def launch_kinds(names):
+    """The kinds of a sequence of launches.  A plane forward transform that
+    follows an inverse one forms the refinement residual (the library times it
+    as such), unless the forward before it did: then it begins the next
+    solve (one refinement step a solve)."""
+    kinds, last, refined = [], None, False
+    for name in names:
+        kind = kernel_kind(name)
+        if kind == "forward" and "k_plane_fwd" in name:
+            refined = last == "inverse" and not refined
+            if refined:
+                kind = "residual"
+        if kind is not None:
+            last = kind
+        kinds.append(kind)
+    return kinds
+
+
 def ncu_summary(csv_path, steps):
     """Per-kernel launches, device time per step and share from an ncu --csv
     launch list (gpu__time_duration.sum) of `bench.py --quick --steps K`
@@ -323,10 +354,8 @@ def ncu_summary(csv_path, steps):
     with open(csv_path) as f:
         lines = [ln for ln in f if ln.startswith('"')]
     agg = {}
-    for r in csv.DictReader(lines):
-        if r["Metric Name"] != "gpu__time_duration.sum":
-            continue
-        kind = kernel_kind(r["Kernel Name"])
+    rows = [r for r in csv.DictReader(lines) if r["Metric Name"] == "gpu__time_duration.sum"]
+    for r, kind in zip(rows, launch_kinds([r["Kernel Name"] for r in rows])):
         if kind is None:
             continue
         short = r["Kernel Name"].replace("void ", "", 1).replace("ibm::", "").split("(")[0]
@@ -758,8 +787,9 @@ def method_bytes(n, precision_bytes, refine, fused=False):
     (read field, write spectrum), pencil (read + write spectrum), inverse
     (read spectrum, write field); a refinement step adds the residual (read
     b and x, write r), a second solve and the read of the updated field.
-    `fused` (the slab path): the residual and the correction's forward x
-    rows are one pass (read b and x, write the spectrum)."""
+    `fused` (the slab path and the plane kernels): the residual and the
+    correction's forward transform, or the x rows of it, are one pass (read b
+    and x, write the spectrum)."""
     pts = n ** 3
     spec = n * n * (n // 2 + 1)
     s = precision_bytes
@@ -809,7 +839,7 @@ def poisson_compare(ibm, torch, n, variants, nb=16, K=40, bc=None, oracle=False)
         lat = [evs[i].elapsed_time(evs[i + 1]) for i in range(K)]
         ms = evs[0].elapsed_time(evs[-1]) / K
         outs[name] = phi[0].double().cpu().numpy()
-        fused = dt == torch.float32 and ref > 0 and slab_path(n, True, bc, env)
+        fused = ref > 0 and fused_residual(n, dt == torch.float32, bc, env)
         mb = method_bytes(n, 4 if dt == torch.float32 else 8, ref if dt == torch.float32 else 0, fused)
         res[name] = {"solves_per_s": 1e3 / ms, "grid_pts_per_s": n ** 3 * 1e3 / ms, "ms": ms,
                      "p50_ms": float(np.percentile(lat, 50)), "p99_ms": float(np.percentile(lat, 99)),

@@ -76,3 +76,31 @@ def test_method_bytes_agrees_with_the_per_kind_count(refine, fused):
     total = sum(bench.solve_kind_bytes(n, esz=4, refine=refine, fused=fused).values())
     assert bench.method_bytes(n, 4, refine, fused=fused) == total
     assert bench.method_bytes(n, 8, refine, fused=fused) == 2 * total
+
+
+def test_residual_fused_where_the_library_forms_it_in_the_transform(monkeypatch):
+    """The slab path and the FP32 plane kernels (cubes up to 128^3 by default)
+    store no residual; the split passes and FP64 do."""
+    import bench
+    for v in ("IBM_SLAB", "IBM_PLANE_MODE"):
+        monkeypatch.delenv(v, raising=False)
+    assert all(bench.fused_residual(n, True) for n in (32, 64, 128, 256))
+    assert bench.fused_residual(128, True, bc=2)            # triply periodic planes
+    assert not bench.fused_residual(192, True)              # split passes
+    assert not bench.fused_residual(256, True, bc=2)
+    assert not bench.fused_residual(256, True, env={"IBM_SLAB": "0"})
+    assert bench.fused_residual(128, True, env={"IBM_SLAB": "0"})
+    assert not bench.fused_residual(128, True, env={"IBM_PLANE_MODE": "0"})
+    assert not any(bench.fused_residual(n, False) for n in (64, 128, 256))
+    # 56.5 B a point at 128^3 (with a stored and reread residual 64.5)
+    assert round(bench.method_bytes(128, 4, 1, True) / 128 ** 3, 1) == 56.5
+
+
+def test_stage_bytes_follow_the_launches():
+    """Four of a stage's five forward transforms read a field; the fifth, timed
+    as the residual, reads b and x."""
+    import bench
+    F, S = _field(128), _spec(128)
+    assert bench.algorithmic_bytes("forward") == 4 * (F + S)
+    assert bench.algorithmic_bytes("residual") == 2 * F + S
+    assert bench.algorithmic_bytes("inverse") == 5 * (S + F) + 4 * F

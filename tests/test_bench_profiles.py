@@ -17,6 +17,19 @@ def test_kernel_kinds():
     assert bench.kernel_kind("void at::native::vectorized_elementwise_kernel<4>()") is None
 
 
+def test_launch_kinds_of_fused_residuals():
+    """Two refined solves by the plane kernels after a stage's three-field
+    solve: the forward transform after a solve's first inverse is the residual
+    pass, the one that begins the next solve is not."""
+    import bench
+    f, p, i = ("void ibm::%s(x)" % k for k in ("k_plane_fwd_ip<128, 128>", "k_pencil_seg<float, 16, 256>",
+                                               "k_plane_inv_ip<128, 128>"))
+    solve = [f, p, i]
+    names = solve + ["void ibm::k_divergence_f32v(x)"] + 2 * (solve + solve)
+    one = ["forward", "pencil", "inverse"]
+    assert bench.launch_kinds(names) == one + ["divergence"] + 2 * (one + ["residual", "pencil", "inverse"])
+
+
 def _launch_csv(path, rows):
     head = '"ID","Kernel Name","Metric Name","Metric Unit","Metric Value"\n'
     with open(path, "w") as f:
