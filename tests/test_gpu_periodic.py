@@ -142,3 +142,28 @@ def test_periodic_every_y_length(ny):
             assert rel_err(host(x), O.helmholtz_solve(b, g, 0.02, O.PERIODIC)) <= tol
         finally:
             ibm.ibm_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("c", [None, 0.02])
+def test_periodic_residual_pass_marches_past_the_wrap(c, monkeypatch):
+    """The split passes' residual pass on a grid whose CTAs march several y planes
+    each (24 column CTAs, some 1,200 resident: chunks of 6 planes, the last
+    one of 4): planes handed down in registers, the wrap at the first plane and
+    in the middle of the last march.  Poisson (c None) and Helmholtz, refined."""
+    monkeypatch.setenv("IBM_PLANE_MODE", "0")
+    shape = (128, 256, 96)
+    b = synth.white_noise(*shape, workload=83, stream=0).astype(np.float32).astype(np.float64)
+    g, plan = _plan(shape, ibm.IBM_FP32_REFINED)
+    try:
+        rhs = dev(b, torch.float32)
+        x = torch.empty_like(rhs)
+        if c is None:
+            ref = O.poisson_solve(b, g, ybc=O.PERIODIC)[0]
+            info = ibm.ibm_poisson_solve(plan, rhs, x, info=True)
+        else:
+            ref = O.helmholtz_solve(b, g, c, O.PERIODIC)
+            info = ibm.ibm_helmholtz_solve(plan, c, ibm.IBM_FIELD_PERIODIC, rhs, x, info=True)
+        assert rel_err(host(x), ref) <= TOL_FP32
+        assert info["rel_residual"] < 1e-3
+    finally:
+        ibm.ibm_plan_destroy(plan)

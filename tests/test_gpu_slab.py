@@ -203,8 +203,9 @@ def test_stream_and_block_residual_agree():
 @pytest.mark.parametrize("nx", [8, 32, 64, 128, 192, 512])
 def test_slab_every_row_length(nx):
     """The x lengths that SLAB_SHAPES leaves out: one or two second-step jobs a
-    thread inside the block's stage (up to 384 points) or beside it (512), and a
-    partial last block (192 points: 21 row pairs a CTA)."""
+    thread inside the block's stage (up to 384 points) or beside it (512).
+    (A block takes 256 / N1 row pairs, a power of two up to 128, and ny nz / 2 pairs
+    of the slab shapes are a multiple of 2048: no block is partial.)"""
     plan, g = _plan((nx, 64, 64), 1)
     try:
         b = (synth.white_noise(nx, 64, 64, workload=57, stream=nx) + 0.25).astype(np.float32)

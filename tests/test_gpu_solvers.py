@@ -483,6 +483,22 @@ def test_plane_kernels_with_residual_inside(shape, monkeypatch):
         ibm.ibm_plan_destroy(plan)
 
 
+@pytest.mark.parametrize("ny", [65, 257])
+def test_poisson_residual_pass_marches_every_plane(ny, monkeypatch):
+    """The same pass without the sigma term (the Poisson operator), its removed
+    mean taken off b on the way: chunks of several planes and a short last one."""
+    monkeypatch.setenv("IBM_PLANE_MODE", "0")
+    g = grid(128, ny, 96)
+    b = synth.white_noise(128, ny, 96, workload=20, stream=ny).astype(np.float32).astype(np.float64) + 0.25
+    plan = _plan(128, ny, 96, g, ibm.IBM_FP32_REFINED)
+    try:
+        x = torch.empty(b.shape, dtype=torch.float32, device="cuda")
+        ibm.ibm_poisson_solve(plan, dev(b, torch.float32), x)
+        assert rel_err(host(x), O.poisson_solve(b, g)[0]) <= TOL_FP32
+    finally:
+        ibm.ibm_plan_destroy(plan)
+
+
 def _compiled(tmp_path, name, source):
     """run() of a small program built against the library's headers."""
     from paper_2406_19920_gb300 import build as B
@@ -490,6 +506,42 @@ def _compiled(tmp_path, name, source):
     src.write_text(source)
     subprocess.run([B._nvcc()] + B._flags() + ["-shared", str(src), "-o", str(lib)], check=True)
     return ctypes.CDLL(str(lib)).run
+
+
+RCP_CU = r"""
+#include "seg.cuh"
+__global__ void k(const double *x, double *r, double *d, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) { r[i] = ibm::rcp<double>(x[i]); d[i] = 1.0 / x[i]; }
+}
+extern "C" int run(const double *x, double *r, double *d, int n) {
+  k<<<(n + 255) / 256, 256>>>(x, r, d, n);
+  const cudaError_t e = cudaDeviceSynchronize();
+  return (int)e;
+}
+"""
+
+
+def test_fp64_reciprocal_within_one_unit(tmp_path):
+    """The sweeps' FP64 reciprocal against 1.0 / x: at most one unit in the last
+    place apart, over random mantissas with exponents of +-300, powers of two
+    and their neighbours, and values next to one."""
+    run = _compiled(tmp_path, "rcp", RCP_CU)
+    r = np.random.default_rng(21)
+    n = 1 << 22
+    p = 2.0 ** np.arange(-300, 301)
+    near = 1.0 + np.arange(-4096, 4097) * 2.0 ** -52
+    x = np.concatenate([(1.0 + r.random(n)) * 2.0 ** r.integers(-300, 301, n), p, np.nextafter(p, np.inf),
+                        np.nextafter(p, 0.0), near])
+    xd = dev(x, torch.float64)
+    got, div = torch.empty_like(xd), torch.empty_like(xd)
+    run.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int]
+    assert run(xd.data_ptr(), got.data_ptr(), div.data_ptr(), len(x)) == 0
+    g, d = host(got), host(div)
+    assert np.array_equal(d, 1.0 / x)
+    units = np.abs(g.view(np.int64) - d.view(np.int64))
+    assert units.max() <= 1, (units.max(), x[units.argmax()])
+    assert (units > 0).mean() < 1e-3
 
 
 DFT_CU = r"""
