@@ -125,7 +125,8 @@ template <typename T, int N> struct ColCfg {
   static constexpr int N1 = TwoStep<N>::N1, N2 = TwoStep<N>::N2;
   // columns per CTA: runs of >= 128 bytes per row; one thread per (column,
   // n1) in step 1, and the same threads take the N2 step-3 DFTs of their
-  // column in turn (about 256 threads, every one busy in both steps)
+  // column in turn (FP32 about 256 threads, FP64 about 64, every one busy in
+  // both steps)
   static constexpr int WMIN = sizeof(T) == 4 ? 16 : 8, WMAX = 64;
   static constexpr int WT0 = (sizeof(T) == 4 ? 256 : 64) / N1;
   static constexpr int WS = (int)(65536 / ((size_t)N * sizeof(cplx<T>)));  // exchange tile <= 64 KB

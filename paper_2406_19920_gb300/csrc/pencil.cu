@@ -820,7 +820,11 @@ cudaError_t launch_pencil(const PencilParams &pp, Ptr3<cplx<T> *> S3, const T *l
     return cudaSuccess;
   }
   // default: the segmented sweep for FP32 (measured faster at 128^3 and
-  // 256^3); FP64 is bound by its divisions and stays on the two-ended sweep
+  // 256^3).  FP64 is bound by its instructions and stays on the two-ended sweep,
+  // which has fewer: 256 x 128 x 128 Poisson 64 against 129 us, the three fields of a
+  // stage 180 against 423, Helmholtz solves at every size; only with few pencils
+  // is the segmented one's shorter chain ahead, in Poisson solves (32 x 128 x 32 39
+  // against 48 us, 32 x 256 x 32 75 against 86)
   if (pp.mode == 4 || (pp.mode == 0 && sizeof(T) == 4 && seg_rows<T>(pp.ny, false) > 0)) {
     // e_k - e+ shrinks by w^2 a row, w + 1 / w = 2 + g / a: with g / a >= 0.4, w^2 <= 0.29 and 16 rows take
     // it below 2^-28

@@ -209,8 +209,10 @@ k_plane_inv(Ptr3<cplx<T> *> S_, Ptr3<T *> out_, Ptr3<const T *> add_, const cplx
 // exchange.  Each thread keeps its job's values in registers over the barrier
 // between a step's reads and its writes, so the CTA needs about the plane's
 // bytes (128 x 128: 72 KB instead of 139) and two CTAs share an SM, each with
-// barriers of its own to wait at.  For lengths up to 128: a job is then at most
-// 16 complex values, and a step has at most two jobs a thread.  Measured against
+// barriers of its own to wait at.  For lengths up to 128, where what a thread
+// holds over a barrier is at most 16 complex values: one job's of x step 1 (N2X),
+// x step 3 (2 N1X) and z step 1 (N2Z), or its RZ3 jobs' of z step 3 (N1Z each; up
+// to three jobs, at z lengths 12 and 48).  Measured against
 // the separate buffers: 128 x 512 x 128 refined solve 163 -> 133 us, 128 x 256 x
 // 128 78 -> 66, 128^3 44.1 -> 43.3, 96^3 32.5 -> 31.5, 48 x 33 x 24 21.8 -> 20.0.
 // --------------------------------------------------------------------------
@@ -222,7 +224,7 @@ template <int NX, int NZ> struct PlaneInPlace {
   static constexpr int mx(int a, int b) { return a > b ? a : b; }
   static constexpr int THREADS = (mx(mx(X1, X3), Z1) + 31) / 32 * 32;
   static constexpr int RZ3 = (Z3 + THREADS - 1) / THREADS;  // rounds of z step 3
-  // CTAs an SM the registers are sized for (at most 56 a thread)
+  // CTAs an SM the registers are sized for (at least 56 a thread)
   static constexpr int CTAS = 1152 / THREADS < 2 ? 2 : 1152 / THREADS > 8 ? 8 : 1152 / THREADS;
   static constexpr int BUF = mx(NZ * P, NZ / 2 * N1X * XPITCH);
   static constexpr size_t bytes = sizeof(float2) * ((size_t)NX + NZ + BUF);

@@ -47,8 +47,9 @@ __device__ __forceinline__ double warp_excl_scan(double v, int lane) {
   return s - v;
 }
 
-// FP64 zero-mode pencil, run by one full warp of a CTA of its own (the last
-// CTA of the pencil grid) concurrently with the other pencils.  Input
+// FP64 zero-mode pencil, run by one full warp of a CTA of its own (the first of
+// k_pencil_seg's grid, the last of the other pencil kernels') or of the kx = 0
+// cluster of k_slab, concurrently with the other pencils.  Input
 // f_j = Re S[j][0][0] (zrhs, written by the forward transform); output
 // zsol[j] (read by the inverse transform).  zs is shared scratch of ny doubles.
 // zrhs, zsol and zs may be one array: each lane reads and writes only its

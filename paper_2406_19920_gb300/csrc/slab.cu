@@ -76,9 +76,9 @@ template <int N> struct RowT {
   // inverse: up to 384 points the exchange area lies in the block's own stage
   // (the spectrum is read into registers before it is written, and it is read
   // into registers before the output rows are): three CTAs share an SM instead of
-  // two at 128 to 256 points, two instead of one at 384, where a pass of 384 x 256
-  // x 256 takes 43.6 instead of 57.2 us (one CTA's chain of copies and barriers
-  // left the SM idle).  At 512 two stages alone leave room for one CTA.
+  // two at 48, 96, 128 and 256 points, two instead of one at 192 and at 384, where a pass of
+  // 384 x 256 x 256 takes 43.6 instead of 57.2 us (one CTA's chain of copies and
+  // barriers left the SM idle).  At 512 two stages alone leave room for one CTA.
   static constexpr bool XSTAGE = N <= 384;
   static constexpr int R3 = (RP * N2 + kRowT - 1) / kRowT;  // step-3 jobs a thread (one in step 1)
   static constexpr size_t o_stage = a128((size_t)N * 8 + (XSTAGE ? 0 : (size_t)RP * QI * 8));  // 128-byte aligned tensor-load targets
@@ -189,7 +189,7 @@ k_rows_fwd_t(const float *__restrict__ in, float2 *__restrict__ S, const float2 
 }
 
 // The refinement's correction right-hand side and its forward x rows in one
-// pass: the residual r = b - A x (residual4, the slab path's wall kinds) of
+// pass: the residual r = b - A x (residual4_rows, the slab path's wall kinds) of
 // the CTA's 2 RP rows into a shared tile (pitch N + 8 floats: the two rows a
 // warp reads in step 1 fall on different banks), then the forward x rows of
 // the tile, whose memory is the exchange area once step 1 has read it into
