@@ -636,7 +636,7 @@ def run_gpu(args):
             bc=ibm.IBM_BC_TRIPLY_PERIODIC)
         out["poisson_128"] = poisson_compare(ibm, torch, NX, (("fp32_refined", ibm.IBM_FP32_REFINED, 1),
                                                               ("fp32_refined_split", ibm.IBM_FP32_REFINED, 1,
-                                                               {"IBM_SLAB": "0"}),
+                                                               {"IBM_SLAB": "0", "IBM_PLANE_MODE": "0"}),
                                                               ("fp64", ibm.IBM_FP64, 0)))
         out["stage_128"] = stage_128(ibm, torch, args, oracle=rank == 0 and not args.no_oracle)
         out["spreading"] = spread_compare(ibm, torch)
