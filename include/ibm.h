@@ -38,6 +38,8 @@
  *   marker is neither interpolated (its U and F are written as 0) nor
  *   spread, and the plan's error word counts it.  ibm_plan_check, and the
  *   next call with a non-NULL info, then return IBM_ERR_ARG with the count.
+ *   x and z are periodic, however far out the marker is; one whose x or z is
+ *   not finite, or 2^46 cells away and more, reads 0 and spreads nothing.
  * Alignment: field pointers must be 16-byte aligned (they are moved with
  *   bulk asynchronous copies); marker arrays need their element alignment.
  * Ownership: all field and marker pointers belong to the caller; the plan
